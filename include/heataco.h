@@ -134,10 +134,11 @@ typedef struct {
 
 /* Execution options of a batch (none of them changes any result). */
 typedef struct {
-    int32_t ants_per_warp;    /* 1, 2 or 4 ants share one warp (8-lane segments), 16 (one ant per
-                                 lane pair) or 32 (one ant per lane); 0 = auto (fused: per
-                                 instance, 4 on one CTA when its table, visited masks and
-                                 coordinates fit in one SM's shared memory, else 2 on a cluster) */
+    int32_t ants_per_warp;    /* 1, 2 or 4 ants share one warp (a lane quad each), 16 (one ant per
+                                 lane pair) or 32 (one ant per lane); 0 = auto (fused: 8,
+                                 on one CTA when the instance's table, visited masks and
+                                 coordinates fit in one SM's shared memory, else on a cluster;
+                                 per-step: as few as keep about 8 warps on every SM) */
     int32_t warps_per_block;  /* construction block size in warps; 0 = auto */
     int32_t use_graph;        /* 1: capture the iteration loop (per-step kernels: 10 iterations
                                  per graph; fused: the group launches) in a CUDA
@@ -255,9 +256,11 @@ int hac_batch_kernel_time(hac_batch *bt, int32_t group, double *ms, int64_t *lau
  * trial_iters iterations took the least device time (CUDA events on
  * `stream`), with use_graph = 1, and that time per iteration in *ms_per_iter
  * (may be NULL).  Candidates: the fused cluster kernel with 2, 4, 16 or 32
- * ants per warp, smallest cluster 1, 2 or 4 CTAs, with and without the
- * 32-entry nearest-unvisited lookup list; the per-step kernels with 1, 2, 4
- * or 16 ants per warp and 4 or 8 warps per block.  No layout changes a result, so the choice
+ * ants per warp or the per-instance choice (0), smallest cluster 1, 2 or 4
+ * CTAs, with and without the 32-entry nearest-unvisited lookup list; the
+ * per-step kernels with 1, 2, 4 or 16 ants per warp and 4 or 8 warps per
+ * block.  The per-instance choice is returned when it is at least 2 % faster
+ * than every other candidate.  No layout changes a result, so the choice
  * is a matter of speed only; the method's parameters (m, k, ...) are never
  * changed.  Uses `workspace` (hac_batch_workspace_size bytes) for each trial
  * in turn; synchronises `stream`.  Candidates an instance does not support
@@ -342,7 +345,7 @@ int hac_solve_batch(const hac_instance *ins, const hac_params *ps, int32_t count
  *                   budget among them each tick
  *   step_ants_per_warp, step_warps_per_block
  *                   layout of that route (0 -> 1 and 8; 1, 2, 4 or 16 and 1..8)
- *   exec            ants_per_warp (0 -> 4; 2, 4, 16 or 32), cluster_log2 (the
+ *   exec            ants_per_warp (0: per request; 2, 4, 16 or 32), cluster_log2 (the
  *                   smallest cluster size, log2), fallback_list (0 or 32);
  *                   fused is implied, the other fields are ignored */
 typedef struct {

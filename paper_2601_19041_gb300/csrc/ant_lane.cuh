@@ -152,7 +152,7 @@ __device__ __forceinline__ void build_tours_lane(const DevInst &I, const Rows &r
                     const unsigned bm = __ballot_sync(FULL_MASK, ok);
                     if (bm) found = __shfl_sync(FULL_MASK, u, __ffs(bm) - 1);
                     if (found < 0 && I.fbl2)
-                        found = lookup2(I.fbl2, scur, lane,
+                        found = lookup2(I.fbl2, scur, lane, n,
                                         [&](int u2) { return (vis_warp[(u2 >> 5) * 32 + L] >> (u2 & 31)) & 1u; });
                 }
                 if (found < 0) {

@@ -175,7 +175,7 @@ __device__ __forceinline__ void build_tours_pair(const DevInst &I, const Rows &r
                 const unsigned bm = __ballot_sync(FULL_MASK, ok);
                 if (bm) found = __shfl_sync(FULL_MASK, u, __ffs(bm) - 1);
                 if (found < 0 && I.fbl2)
-                    found = lookup2(I.fbl2, scur, lane, [&](int u2) { return (sv[16 * (u2 >> 5)] >> (u2 & 31)) & 1u; });
+                    found = lookup2(I.fbl2, scur, lane, n, [&](int u2) { return (sv[16 * (u2 >> 5)] >> (u2 & 31)) & 1u; });
             }
             if (found < 0) {
                 float bk = __int_as_float(0x7f800000);

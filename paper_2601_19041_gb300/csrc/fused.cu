@@ -20,6 +20,7 @@
 
 #include "ant_lane.cuh"
 #include "ant_pair.cuh"
+#include "ant_quad.cuh"
 #include "iter.cuh"
 #include "threeopt.cuh"
 
@@ -48,11 +49,18 @@ __host__ __device__ inline size_t fused_table_bytes(int rows_cap, int kp_cap)
     return ch + ix;
 }
 
-// APW ants per warp: 2 or 4 (warp segments, ant.cuh), 16 (one ant per lane
-// pair, ant_pair.cuh, NG slot groups per lane) or 32 (one ant per lane,
-// ant_lane.cuh, NG candidate groups).  Shared memory per CTA:
-//   choice rows (FP32) | candidate ids (uint16) | visited masks |
-//   coordinates (optional) | lookup lists (uint16, optional)
+// visited masks, rounded so that what follows them is 16-byte aligned
+__host__ __device__ inline size_t fused_vis_bytes(int warps, int apw, int stride)
+{
+    return ((size_t)warps * apw * stride * 4 + 15) & ~(size_t)15;
+}
+
+// APW 8: one ant per lane quad, A.apw <= 8 ants per warp (ant_quad.cuh, NG
+// candidate groups); 16: one ant per lane pair (ant_pair.cuh, NG slot groups
+// per lane); 32: one ant per lane (ant_lane.cuh, NG candidate groups).
+// Shared memory per CTA:
+//   choice rows (FP32) | candidate ids (uint16) | rings (APW 8) | visited
+//   masks | coordinates (optional) | lookup lists (uint16, optional)
 template <int APW, int NG, int CLOG>
 __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
 {
@@ -68,10 +76,11 @@ __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
     extern __shared__ __align__(16) unsigned char smem[];
     float *sch = reinterpret_cast<float *>(smem);
     uint16_t *sidx = reinterpret_cast<uint16_t *>(smem + (size_t)A.rows_cap * A.kp_cap * 4);
-    unsigned *svis = reinterpret_cast<unsigned *>(smem + fused_table_bytes(A.rows_cap, A.kp_cap));
-    float2 *sxy = reinterpret_cast<float2 *>(smem + fused_table_bytes(A.rows_cap, A.kp_cap) +
-                                             (size_t)A.warps * APW * A.stride * 4);
-    uint16_t *slist = reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(sxy) + (size_t)A.xy_cap * 8);
+    const int apw = APW == 8 ? A.apw : APW;   // ants per warp
+    uint32_t *sring = reinterpret_cast<uint32_t *>(smem + fused_table_bytes(A.rows_cap, A.kp_cap));
+    unsigned *svis = sring + (APW == 8 ? A.warps * apw * QRING_W : 0);
+    float2 *sxy = reinterpret_cast<float2 *>(reinterpret_cast<unsigned char *>(svis) + fused_vis_bytes(A.warps, apw, A.stride));
+    uint16_t *slist = reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(sxy) + (((size_t)A.xy_cap * 8 + 15) & ~(size_t)15));
 
     const int n = I.n, kp = I.k_pad, m = I.m;
     const int R = (n + C - 1) >> CLOG;   // local rows: i = rank + C*l
@@ -101,10 +110,12 @@ __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
             const int v = i < n ? I.fbl[(size_t)i * FBL + k] : -1;
             slist[e] = v < 0 ? (uint16_t)0xffff : (uint16_t)v;
         }
-    ClusterRows<CLOG> rows;
-    rows.idx_base = (uint32_t)__cvta_generic_to_shared(sidx);
-    rows.ch_base = (uint32_t)__cvta_generic_to_shared(sch);
-    rows.kp = kp;
+    const uint32_t idx_base = (uint32_t)__cvta_generic_to_shared(sidx), ch_base = (uint32_t)__cvta_generic_to_shared(sch);
+    const ClusterRows<CLOG> rows{idx_base, ch_base, kp};
+    __shared__ __align__(16) unsigned qpad[6];   // a quad lane's record of padding slots
+    if (threadIdx.x < 6) qpad[threadIdx.x] = threadIdx.x < 4 ? 0u : (unsigned)n * 0x10001u;
+    const ClusterQuadRows<NG == 8 ? 2 : 1, NG == 5, CLOG> qrows(idx_base, ch_base, (uint32_t)__cvta_generic_to_shared(qpad),
+                                                                kp, threadIdx.x & 3);
     const ClusterList<CLOG> clist{list_shared ? (uint32_t)__cvta_generic_to_shared(slist) : 0u};
     const GlobalList glist{I.fbl};
     const int t0 = st->t;
@@ -114,10 +125,11 @@ __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
     const int apc = (m + C - 1) >> CLOG;   // ants per CTA
     const int a_lo = rank * apc, a_hi = min(m, a_lo + apc);
     const float omega = __double2float_rn(__dsub_rn(1.0, I.rho));
-    unsigned *vis_w = svis + (size_t)wib * APW * A.stride;
+    unsigned *vis_w = svis + (size_t)wib * apw * A.stride;
+    uint32_t *ring_w = sring + wib * apw * QRING_W;
 
     for (int t = t0; t < t_end; ++t) {
-        const int a_first = a_lo + wib * APW;
+        const int a_first = a_lo + wib * apw;
         if (a_first < a_hi) {
             if constexpr (APW == 32) {
                 if (list_shared) build_tours_lane<NG>(I, rows, clist, t, a_first, a_hi, vis_w, xy_scan);
@@ -126,18 +138,19 @@ __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
                 if (list_shared) build_tours_pair<NG>(I, rows, clist, t, a_first, a_hi, vis_w, A.stride, xy_scan);
                 else build_tours_pair<NG>(I, rows, glist, t, a_first, a_hi, vis_w, A.stride, xy_scan);
             } else {
+                constexpr int NGL = NG == 8 ? 2 : 1;
+                constexpr bool TAIL = NG == 5;
+                const int a_end = min(a_first + apw, a_hi);
                 if (list_shared)
-                    build_tours<APW, ClusterRows<CLOG>, ClusterList<CLOG>, NG>(I, rows, clist, t, a_first, a_hi,
-                                                                             vis_w, A.stride, xy_scan);
+                    build_tours_quad<NGL, TAIL>(I, qrows, clist, t, a_first, a_end, vis_w, A.stride, ring_w, xy_scan);
                 else
-                    build_tours<APW, ClusterRows<CLOG>, GlobalList, NG>(I, rows, glist, t, a_first, a_hi, vis_w,
-                                                                      A.stride, xy_scan);
+                    build_tours_quad<NGL, TAIL>(I, qrows, glist, t, a_first, a_end, vis_w, A.stride, ring_w, xy_scan);
             }
         }
         __syncthreads();
-        fallback_distances(I, a_lo, a_hi);     // this CTA's ants only: no cluster barrier needed
         if (I.local_search == 2 || I.local_search == 4) {   // Algorithm 1's local search on every ant
-            for (int a = a_first; a < min(a_first + APW, a_hi); ++a) {   // each warp its own
+            ant_lengths(I, a_lo, a_hi, false);
+            for (int a = a_first; a < min(a_first + apw, a_hi); ++a) {   // each warp its own
                 int32_t *tour = I.tours + (size_t)a * n;
                 if (I.local_search == 4) warp_three_opt(I, tour, ls_ant(I, a));
                 else warp_two_opt_any(I, tour, ls_ant(I, a));
@@ -146,7 +159,7 @@ __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
             }
             __syncthreads();
         } else {
-            ant_lengths(I, a_lo, a_hi);
+            ant_lengths(I, a_lo, a_hi, true);      // this CTA's ants only: no cluster barrier needed
         }
         __threadfence();
         cl.sync();
@@ -216,14 +229,14 @@ __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
 // ------------------------------------------------------------ host side
 
 template <typename Kern>
-static cudaError_t launch_cluster(Kern kern, int clog, const FusedArgs &A, int clusters, int warps,
+static cudaError_t launch_cluster(Kern kern, int clog, const FusedArgs &A, int clusters, int block_warps,
                                   size_t smem, cudaStream_t s, bool after_resident)
 {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters << clog), 1, 1);
-    cfg.blockDim = dim3((unsigned)(warps * 32), 1, 1);
+    cfg.blockDim = dim3((unsigned)(block_warps * 32), 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -243,22 +256,22 @@ static cudaError_t launch_cluster(Kern kern, int clog, const FusedArgs &A, int c
 size_t fused_smem_bytes(int rows_cap, int kp_cap, int warps, int apw, int stride, int xy_cap,
                         int list_rows)
 {
-    return fused_table_bytes(rows_cap, kp_cap) + (size_t)warps * apw * stride * 4 + (size_t)xy_cap * 8 +
-           (size_t)list_rows * FBL * 2;
+    return fused_table_bytes(rows_cap, kp_cap) + (apw <= 8 ? (size_t)warps * apw * QRING_W * 4 : 0) +
+           fused_vis_bytes(warps, apw, stride) + (((size_t)xy_cap * 8 + 15) & ~(size_t)15) + (size_t)list_rows * FBL * 2;
 }
 
 cudaError_t launch_fused(const DevInst *d_inst, const int32_t *d_order, const int32_t *d_iters,
-                         int clusters, int clog, int apw, int warps, int rows_cap, int kp_cap, int stride,
-                         int xy_cap, int list_rows, int iters, cudaStream_t s, bool after_resident)
+                         int clusters, int clog, int apw, int warps, int block_warps, int rows_cap, int kp_cap,
+                         int stride, int xy_cap, int list_rows, int iters, cudaStream_t s, bool after_resident)
 {
     FusedArgs A{d_inst, d_order, d_iters, iters, rows_cap, kp_cap, stride, warps, apw, xy_cap, list_rows};
     const size_t smem = fused_smem_bytes(rows_cap, kp_cap, warps, apw, stride, xy_cap, list_rows);
 #define CLUSTER_SWITCH(APWV, NGV) \
     switch (clog) { \
-    case 0: return launch_cluster(k_fused<APWV, NGV, 0>, 0, A, clusters, warps, smem, s, after_resident); \
-    case 1: return launch_cluster(k_fused<APWV, NGV, 1>, 1, A, clusters, warps, smem, s, after_resident); \
-    case 2: return launch_cluster(k_fused<APWV, NGV, 2>, 2, A, clusters, warps, smem, s, after_resident); \
-    default: return launch_cluster(k_fused<APWV, NGV, 3>, 3, A, clusters, warps, smem, s, after_resident); }
+    case 0: return launch_cluster(k_fused<APWV, NGV, 0>, 0, A, clusters, block_warps, smem, s, after_resident); \
+    case 1: return launch_cluster(k_fused<APWV, NGV, 1>, 1, A, clusters, block_warps, smem, s, after_resident); \
+    case 2: return launch_cluster(k_fused<APWV, NGV, 2>, 2, A, clusters, block_warps, smem, s, after_resident); \
+    default: return launch_cluster(k_fused<APWV, NGV, 3>, 3, A, clusters, block_warps, smem, s, after_resident); }
     if (apw == 32) {
         const int G = kp_cap / 4;
         if (G <= 3) { CLUSTER_SWITCH(32, 3) }
@@ -271,13 +284,10 @@ cudaError_t launch_fused(const DevInst *d_inst, const int32_t *d_order, const in
         if (G <= 6) { CLUSTER_SWITCH(16, 3) }
         CLUSTER_SWITCH(16, 4)
     }
-    // 2 or 4 ants per warp: the group totals are gathered (5 groups for k <= 20, else 8)
-    if (apw == 2) {
-        if (kp_cap <= 20) { CLUSTER_SWITCH(2, 5) }
-        CLUSTER_SWITCH(2, 8)
-    }
-    if (kp_cap <= 20) { CLUSTER_SWITCH(4, 5) }
-    CLUSTER_SWITCH(4, 8)
+    // one ant per quad: kp_cap/4 slot groups
+    if (kp_cap <= 16) { CLUSTER_SWITCH(8, 4) }
+    if (kp_cap <= 20) { CLUSTER_SWITCH(8, 5) }
+    CLUSTER_SWITCH(8, 8)
 #undef CLUSTER_SWITCH
 }
 

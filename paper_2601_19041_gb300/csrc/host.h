@@ -30,6 +30,19 @@ constexpr int ROWS_PER_BLOCK = 8;      // matches the row kernels (8 warps, a ro
 constexpr int SLOTS_PER_BLOCK = 1024;  // matches the slot kernels
 constexpr int GRAPH_CHUNK = 10;        // iterations per captured graph
 constexpr int FBL_LEN = FBL1_LEN;      // nearest-unvisited lookup list
+constexpr int GPU_SMS = 152;           // SMs of a GB300
+
+// Ants per warp of the per-step kernels when the caller leaves it open: as few
+// as keep about 8 warps on every SM.  A warp's ants wait for each other's
+// nearest-unvisited steps, and up to 8 warps per SM do not wait for issue
+// slots (16 x n = 5000, k = 20, 20 iterations end to end: 66.9 / 66.8 / 73.5 /
+// 83.9 ms with 1 / 2 / 4 / 8 ants per warp; one n = 500 instance, 100
+// iterations: 24.7 / 24.5 / 26.4 / 31.3 ms).
+inline int step_ants_per_warp(long long ants)
+{
+    const long long a = (ants + 8 * GPU_SMS - 1) / (8 * GPU_SMS);
+    return a < 1 ? 1 : a > 8 ? 8 : (int)a;
+}
 
 struct Arena {
     size_t off = 0;
@@ -278,7 +291,7 @@ inline int plan_batch(const hac_instance *ins, const hac_params *ps, int count, 
 
 struct FusedGroup {
     int clog = 0, apw = 4, count = 0, order_off = 0;
-    int rows_cap = 0, kp_cap = 0, stride = 0, warps = 0, xy_cap = 0, list_rows = 0;
+    int rows_cap = 0, kp_cap = 0, stride = 0, warps = 0, block_warps = 0, xy_cap = 0, list_rows = 0;
 };
 
 // pointers of the zero-initialised part of one instance
@@ -354,12 +367,13 @@ inline int upload_inputs(const DevInst &D, const hac_instance &in, const Sizes &
 // Groups the given instances by layout: ants per warp and cluster size (the
 // fewest CTAs whose shared memory holds the instance's share of the
 // candidate table and visited masks, at least 2^clog_min), each group ordered
-// by decreasing work.  apw = 0 chooses per instance ("mixed"): 4 ants per warp
-// on one CTA where the instance fits one with its coordinates and lookup
-// lists (many ants per SM), else 2 ants per warp on the smallest cluster that
-// holds it (fewer ants per SM, a shorter step for the large instances that
-// bound the batch).  `order` lists
-// instance indices group after group.
+// by decreasing work.  apw = 0 stands for 8 ants per warp, on one CTA where the
+// instance fits one with its coordinates, else on the smallest cluster that
+// holds it.  8 ants per warp keep the fewest warps waiting for issue slots: 64
+// ants on one SM take 839 cycles per step at n = 500 on 8 warps and 1127 on 16;
+// 128 instances of n ~ U{500..2000} decode in 250 ms, in 263 ms with 4 ants per
+// warp on one SM and in 275 ms with 4 ants per warp on the clusters.
+// `order` lists instance indices group after group.
 inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &members, int apw,
                        int clog_min, int fallback_list, std::vector<FusedGroup> &groups,
                        std::vector<int32_t> &order)
@@ -386,24 +400,23 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
             // the rest of the batch, whose makespan is otherwise bound by the
             // SM time of the clusters rather than by its longest instance.
             const Sizes &z = zs[members[q]];
-            if (clog_min == 0 && fits(q, 0, 4, rows, warps) &&
-                fused_smem_bytes(rows, z.kp, warps, 4, (z.n + 32) / 32, z.n, 0) <= FUSED_SMEM_LIMIT) {
+            qapw[q] = 8;
+            if (clog_min == 0 && fits(q, 0, 8, rows, warps) &&
+                fused_smem_bytes(rows, z.kp, warps, 8, (z.n + 32) / 32, z.n, 0) <= FUSED_SMEM_LIMIT) {
                 clog[q] = 0;
-                qapw[q] = 4;
                 continue;
             }
-            qapw[q] = 2;
         }
         for (int cl = clog_min; cl <= 3; ++cl)
             if (fits(q, cl, qapw[q], rows, warps)) { clog[q] = cl; break; }
         if (clog[q] < 0) return HAC_EUNSUPPORTED;
     }
-    const int apws[4] = {2, 4, 16, 32};
+    const int apws[5] = {2, 4, 8, 16, 32};
     for (;;) {   // group caps may exceed the limit when members differ: move a group up
         groups.clear();
         bool again = false;
         for (int cl = 0; cl <= 3 && !again; ++cl)
-            for (int ai = 0; ai < 4 && !again; ++ai) {
+            for (int ai = 0; ai < 5 && !again; ++ai) {
                 const int a = apws[ai];
                 FusedGroup G;
                 G.clog = cl;
@@ -420,6 +433,10 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
                     G.warps = std::max(G.warps, warps);
                 }
                 if (!G.count) continue;
+                // the warps beyond those that build tours share the rest of an
+                // iteration; 16 fill the SM's registers, so a group with more
+                // CTAs than SMs takes 8 and lets two CTAs share an SM
+                G.block_warps = std::max(G.warps, a > 8 ? 1 : (G.count << cl) > GPU_SMS ? 8 : 16);
                 const size_t base = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, 0, 0);
                 if (base > FUSED_SMEM_LIMIT) {
                     if (cl == 3) return HAC_EUNSUPPORTED;
@@ -483,7 +500,7 @@ inline cudaError_t launch_groups(const DevInst *d_inst, const int32_t *d_order, 
     for (size_t g = 0; g < groups.size(); ++g) {
         const FusedGroup &G = groups[g];
         cudaError_t e = launch_fused(d_inst, d_order + G.order_off, d_iters ? d_iters + G.order_off : nullptr,
-                                     G.count, G.clog, G.apw, G.warps,
+                                     G.count, G.clog, G.apw, G.warps, G.block_warps,
                                      G.rows_cap, G.kp_cap, G.stride, G.xy_cap, G.list_rows, iters, s, g > 0);
         if (e != cudaSuccess && err == cudaSuccess) err = e;
     }

@@ -25,55 +25,19 @@ __device__ __forceinline__ size_t step_ix(const DevInst &I, int a, int s)
     return (size_t)a * I.tour_sa + (size_t)s * I.tour_ss;
 }
 
-// d of the listed nearest-unvisited steps and of the closing edge of ants
-// [a_lo, a_hi) (at most 1024 ants): the CTA flattens all (ant, entry) pairs
-// and every thread takes several, so many FP64 square roots are in flight.
-// Call with all threads of the block.
-__device__ __forceinline__ void fallback_distances(const DevInst &I, int a_lo, int a_hi)
+// d of ant a's listed nearest-unvisited steps and of its closing edge, into
+// dstep (whole warp, an entry per lane); returns their number.  The warp that
+// sums the ant's length calls it, so no barrier wider than the warp is needed.
+__device__ __forceinline__ int warp_fallback_distances(const DevInst &I, int a)
 {
-    __shared__ int off[1025];
-    const int n = I.n, na = a_hi > a_lo ? a_hi - a_lo : 0;   // a CTA may own no ant
-    // exclusive prefix over (fallbacks + 1 closing edge) per ant
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int q = 0; q < na; ++q) { off[q] = acc; acc += I.fbcnt[a_lo + q] + 1; }
-        off[na] = acc;
+    const int lane = threadIdx.x & 31, n = I.n, cnt = I.fbcnt[a];
+    const int32_t *fbs = I.fbs + (size_t)a * n;
+    for (int e = lane; e <= cnt; e += 32) {
+        const int s = e < cnt ? fbs[e] : 0;            // 0: the closing edge
+        const int from = I.tours[step_ix(I, a, s ? s - 1 : n - 1)], to = I.tours[step_ix(I, a, s)];
+        I.dstep[step_ix(I, a, s)] = dist64(I, from, to);
     }
-    __syncthreads();
-    const int total = off[na];
-    for (int e0 = threadIdx.x; e0 < total; e0 += 4 * blockDim.x) {
-        int from[4], to[4];
-        size_t ix[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int e = e0 + k * blockDim.x;
-            ix[k] = (size_t)-1;
-            if (e >= total) continue;
-            int lo = 0, hi = na - 1;           // ant of entry e: last q with off[q] <= e
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (off[mid] <= e) lo = mid; else hi = mid - 1;
-            }
-            const int a = a_lo + lo, kk = e - off[lo];
-            if (kk < I.fbcnt[a]) {
-                const int s = I.fbs[(size_t)a * n + kk];
-                from[k] = I.tours[step_ix(I, a, s - 1)];
-                to[k] = I.tours[step_ix(I, a, s)];
-                ix[k] = step_ix(I, a, s);
-            } else {                           // closing edge, stored at step 0
-                from[k] = I.tours[step_ix(I, a, n - 1)];
-                to[k] = I.tours[step_ix(I, a, 0)];
-                ix[k] = step_ix(I, a, 0);
-            }
-        }
-        double d[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) d[k] = ix[k] != (size_t)-1 ? dist64(I, from[k], to[k]) : 0.0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) if (ix[k] != (size_t)-1) I.dstep[ix[k]] = d[k];
-    }
-    if (threadIdx.x == 0) atomicAdd(&I.st->n_fallback, (unsigned long long)(total - na));
-    __syncthreads();
+    return cnt;
 }
 
 // lengths of NA ants at once (whole warp; results in every lane): the loops
@@ -136,24 +100,34 @@ __device__ __forceinline__ void warp_ant_lengths(const DevInst &I, const int (&a
     for (int h = 0; h < NA; ++h) out[h] = P[h];
 }
 
-// lengths of ants [a_lo, a_hi): one warp per ant, two ants per warp at a time
-__device__ __forceinline__ void ant_lengths(const DevInst &I, int a_lo, int a_hi)
+// lengths of ants [a_lo, a_hi): one warp per ant, two ants per warp at a
+// time (without `sums`, the nearest-unvisited steps are counted only: local
+// search on every ant recomputes the lengths)
+__device__ __forceinline__ void ant_lengths(const DevInst &I, int a_lo, int a_hi, bool sums)
 {
     const int wib = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    int fb = 0;
     for (int a = a_lo + wib; a < a_hi; a += 2 * nw) {
         const int b = a + nw;
-        if (b < a_hi) {
+        if (!sums) {
+            fb += I.fbcnt[a] + (b < a_hi ? I.fbcnt[b] : 0);
+        } else if (b < a_hi) {
             const int ab[2] = {a, b};
             double L[2];
+            fb += warp_fallback_distances(I, a) + warp_fallback_distances(I, b);
+            __syncwarp();
             warp_ant_lengths<2>(I, ab, L);
             if (lane == 0) { I.lens[a] = L[0]; I.lens[b] = L[1]; }
         } else {
             const int a1[1] = {a};
             double L[1];
+            fb += warp_fallback_distances(I, a);
+            __syncwarp();
             warp_ant_lengths<1>(I, a1, L);
             if (lane == 0) I.lens[a] = L[0];
         }
     }
+    if (lane == 0 && fb) atomicAdd(&I.st->n_fallback, (unsigned long long)fb);
 }
 
 // length of an explicit tour (T_NN, T_ib after 2-opt), whole warp, same order

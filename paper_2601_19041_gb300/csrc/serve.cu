@@ -299,7 +299,7 @@ int enqueue_step_route(hac_server *sv, const std::vector<int> &mem, int par)
     int4 *hw = sv->h_swarp[par];
     int2 *hs = sv->h_sslot[par];
     size_t nw = 0, ns = 0;
-    int it = sv->cfg.iters_per_tick, max_n = 0, max_kp = 0;
+    int it = sv->cfg.iters_per_tick, max_n = 0, max_kp = 0, max_m = 0;
     bool any_ls = false;
     int ls_all_m = 0;
     for (size_t b = 0; b < mem.size(); ++b) {
@@ -311,6 +311,7 @@ int enqueue_step_route(hac_server *sv, const std::vector<int> &mem, int par)
         it = std::min(it, tick_iters(sv, S));
         max_n = std::max(max_n, S.z.n);
         max_kp = std::max(max_kp, S.z.kp);
+        max_m = std::max(max_m, S.z.m);
         any_ls |= S.z.ls != 0;
         if (S.z.ls == 2 || S.z.ls == 4) ls_all_m = std::max(ls_all_m, S.z.m);
     }
@@ -323,7 +324,7 @@ int enqueue_step_route(hac_server *sv, const std::vector<int> &mem, int par)
     CK(cudaMemcpyAsync(sv->d_sslot[par], hs, ns * sizeof(int2), cudaMemcpyHostToDevice, ss));
     for (int q = 0; q < it; ++q) {
         sv->launches += launch_construct(sv->d_sinst[par], sv->d_swarp[par], (int)nw, apw,
-                                         sv->sex.warps_per_block, max_n, max_kp, count, ss);
+                                         sv->sex.warps_per_block, max_n, max_kp, max_m, count, ss);
         sv->launches += launch_iteration_tail(sv->d_sinst[par], count, sv->d_sslot[par], (int)ns, any_ls, max_n,
                                               ls_all_m, ss);
     }
@@ -359,8 +360,7 @@ int hac_server_create(const hac_server_cfg *cfg, void *workspace, size_t ws_byte
     const int s_wpb = c.step_warps_per_block ? c.step_warps_per_block : 8;
     if ((s_apw != 1 && s_apw != 2 && s_apw != 4 && s_apw != 16) || s_wpb < 1 || s_wpb > 8) return HAC_EINVAL;
     hac_exec ex = c.exec;
-    if (ex.ants_per_warp == 0) ex.ants_per_warp = 4;
-    if (ex.ants_per_warp != 2 && ex.ants_per_warp != 4 && ex.ants_per_warp != 16 && ex.ants_per_warp != 32)
+    if (ex.ants_per_warp != 0 && ex.ants_per_warp != 2 && ex.ants_per_warp != 4 && ex.ants_per_warp != 16 && ex.ants_per_warp != 32)
         return HAC_EINVAL;
     if (ex.fallback_list != 0 && ex.fallback_list != FBL_LEN) return HAC_EINVAL;
     if (ex.cluster_log2 < 0 || ex.cluster_log2 > 3) return HAC_EINVAL;
