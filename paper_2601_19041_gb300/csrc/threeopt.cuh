@@ -18,9 +18,25 @@
 //   cleared and a is examined again; a city without a move gets its bit set.
 //   Gains are FP64, each operation rounded once, in the order written.
 //
-// Parallelism: one t5 per lane (both t6 of it), the first lane with an
-// admissible move wins; the g1 values of all t3 are computed at once, one
-// per lane.
+// FP32 scan.  As in the 2-opt, gains are first estimated from FP32 distances
+// (ls_d32, each within 4 units of 2^-24 of the FP64 one): with a band of 4e-6
+// of the terms' sum (six terms and five additions err by less than 6e-7 of
+// it) an estimate outside the band decides, and g1 > 0 and g2 > 0 likewise.
+// ls3_scan tests one city: its (direction, t3, t4) pairs with g1 possibly
+// positive are dealt to the lanes, each lane running through its pair's t5
+// and t6 in order; the first pair with a possible move gives the first
+// possible move of the city.  It is applied when every decision on the way
+// was outside the band; otherwise ls3_examine searches the city again in
+// FP64 (one t5 per lane).  FP64 is slow on this GPU (a dependent add takes about
+// 100 cycles with its use, a distance several hundred): with FP64 alone one
+// search took 47 ms (n = 500, 10-node lists, m = 32, start tour from the ants),
+// and 8 iterations of 32 such instances 469 ms end to end; with the scan and the
+// helper warps they take 41 ms.
+//
+// Helper warps (a block of several warps, see twoopt.cuh) test the next clear
+// cities in tour order at the same time, one per warp: cities before the first
+// one with a possible move have none, and testing them changes nothing.  They
+// also share long middle rewrites.
 //
 // Applying a move: the removed edges sit at tour positions e_0 < e_1 (< e_2)
 // (edge e joins tour[e] and tour[e+1 mod n]); positions outside
@@ -62,78 +78,71 @@ __device__ __forceinline__ int ls3_edge(const LsMem &M, int n, int u, int v)
 // Checks that removing the r edges {c[2k], c[2k+1]} and adding the r edges
 // {c[2k+1], c[(2k+2) mod 2r]} (that is (t2,t3), (t4,t5), (t6,t1) for
 // c = t1..t6, or (t2,t3), (t4,t1) for r = 2) leaves one cycle; plans it.
+// The removed edges, sorted by position, have 2r endpoint slots: 2q is
+// tour[e_q] and 2q + 1 is tour[e_q + 1].  The fixed part ends at slot 0 and
+// starts at slot 2r - 1; middle segment j runs from slot 2j + 1 to slot 2j + 2.
+// The added edges pair the slots; the pairing (a nibble per slot) is walked
+// from slot 0 through every middle segment to slot 2r - 1.
 template <int R>
 __device__ __forceinline__ bool ls3_plan(const LsMem &M, int n, const int (&c)[2 * R], Xchg &X)
 {
     int e[R];
+    bool ok = true;
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         e[k] = ls3_edge(M, n, c[2 * k], c[2 * k + 1]);
-        if (e[k] < 0) return false;
+        ok &= e[k] >= 0;
     }
-    // rank of each removed edge by position
-    int rk[R];
+    if (!ok) return false;
+    int slot[2 * R];
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         int q = 0;
 #pragma unroll
-        for (int l = 0; l < R; ++l) {
-            if (l != k && e[l] == e[k]) return false;
-            q += e[l] < e[k];
-        }
-        rk[k] = q;
+        for (int l = 0; l < R; ++l) q += e[l] < e[k];
+        const int u = M.tour[e[k]];
+        slot[2 * k] = 2 * q + (u == c[2 * k] ? 0 : 1);
+        slot[2 * k + 1] = 2 * q + (u == c[2 * k + 1] ? 0 : 1);
     }
-    // endpoint slot of city c[i] on its removed edge k = i/2: 2*rank + 0 when it
-    // is tour[e] (end of the part before the edge), + 1 when it is tour[e+1]
-    int slot[2 * R];
-#pragma unroll
-    for (int i = 0; i < 2 * R; ++i) {
-        const int k = i >> 1;
-        slot[i] = 2 * rk[k] + (M.tour[e[k]] == c[i] ? 0 : 1);
-    }
-    // added edge i joins slot[2i+1] and slot[(2i+2) mod 2R]
-    int partner[2 * R];
-#pragma unroll
-    for (int i = 0; i < 2 * R; ++i) partner[i] = -1;
+    unsigned pair = 0u, seen = 0u;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
         const int u = slot[2 * i + 1], v = slot[(2 * i + 2) % (2 * R)];
-        if (u == v || partner[u] >= 0 || partner[v] >= 0) return false;
-        partner[u] = v;
-        partner[v] = u;
+        pair |= ((unsigned)v << (4 * u)) | ((unsigned)u << (4 * v));
+        seen |= (1u << u) | (1u << v);
     }
-    // walk from the end of the fixed part (slot 0) until its start (slot 2R-1);
-    // middle segment j starts at slot 2j+1 and ends at slot 2j+2
-    bool used[R - 1];
-#pragma unroll
-    for (int j = 0; j < R - 1; ++j) used[j] = false;
-    int cur = 0, cnt = 0;
-#pragma unroll
-    for (int step = 0; step < R; ++step) {
-        const int s = partner[cur];
-        if (s == 2 * R - 1) break;
-        if (s == 0) return false;
-        const bool back = (s & 1) == 0;
-        const int j = back ? (s >> 1) - 1 : (s - 1) >> 1;
-        if (j < 0 || j >= R - 1 || used[j] || cnt >= R - 1) return false;
-        used[j] = true;
-        X.seg[cnt] = j;
-        X.rev[cnt] = back ? 1 : 0;
-        ++cnt;
-        cur = back ? 2 * j + 1 : 2 * j + 2;
-    }
-    if (cnt != R - 1 || partner[cur] != 2 * R - 1) return false;
+    if (seen != (1u << (2 * R)) - 1u) return false;   // equal edges, or a slot taken twice
+    auto partner = [&](int s) { return (int)((pair >> (4 * s)) & 15u); };
+    const int s0 = partner(0);
+    if (s0 == 2 * R - 1) return false;                // the middle would be left out
+    const int j0 = (s0 - 1) >> 1, x0 = ((s0 - 1) ^ 1) + 1;   // its segment and the segment's other end
     X.r = R;
-    // sorted positions
-#pragma unroll
-    for (int k = 0; k < R; ++k) X.e[rk[k]] = e[k];
-    return true;
+    X.seg[0] = j0;
+    X.rev[0] = (s0 & 1) ? 0 : 1;
+    const int s1 = partner(x0);
+    if constexpr (R == 2) {
+        X.e[0] = min(e[0], e[1]);
+        X.e[1] = max(e[0], e[1]);
+        X.e[2] = 0;
+        X.seg[1] = 0;
+        X.rev[1] = 0;
+        return s1 == 3;
+    } else {
+        if (s1 == 5 || ((s1 - 1) >> 1) == j0) return false;
+        X.seg[1] = (s1 - 1) >> 1;
+        X.rev[1] = (s1 & 1) ? 0 : 1;
+        X.e[0] = min(min(e[0], e[1]), e[2]);
+        X.e[2] = max(max(e[0], e[1]), e[2]);
+        X.e[1] = e[0] + e[1] + e[2] - X.e[0] - X.e[2];
+        return partner(((s1 - 1) ^ 1) + 1) == 5;
+    }
 }
 
-// rewrites the middle positions of the planned exchange (whole warp)
-__device__ __forceinline__ void ls3_apply(const LsMem &M, const Xchg &X)
+// the share of thread tid of nth in rewriting the middle positions of an
+// exchange: phase 0 collects the new middle in the scratch array, phase 1
+// writes it back (a barrier between them)
+__device__ __forceinline__ void ls3_rewrite_part(const LsMem &M, const Xchg &X, int tid, int nth, int phase)
 {
-    const int lane = threadIdx.x & 31;
     int32_t *tmp = reinterpret_cast<int32_t *>(M.el);
     const int lo = X.e[0] + 1;
     const int a0 = X.e[X.seg[0]] + 1, b0 = X.e[X.seg[0] + 1];
@@ -141,19 +150,59 @@ __device__ __forceinline__ void ls3_apply(const LsMem &M, const Xchg &X)
     int a1 = 0, b1 = -1;
     if (X.r == 3) { a1 = X.e[X.seg[1]] + 1; b1 = X.e[X.seg[1] + 1]; }
     const int total = len0 + (b1 - a1 + 1);
-    __syncwarp();
-    for (int w = lane; w < total; w += 32) {
-        int src;
-        if (w < len0) src = X.rev[0] ? b0 - w : a0 + w;
-        else src = X.rev[1] ? b1 - (w - len0) : a1 + (w - len0);
-        tmp[w] = M.tour[src];
+    for (int w = tid; w < total; w += nth) {
+        if (phase == 0) {
+            int src;
+            if (w < len0) src = X.rev[0] ? b0 - w : a0 + w;
+            else src = X.rev[1] ? b1 - (w - len0) : a1 + (w - len0);
+            tmp[w] = M.tour[src];
+        } else {
+            const int c = tmp[w];
+            M.tour[lo + w] = c;
+            M.pos[c] = lo + w;
+        }
     }
+}
+
+constexpr int LS3_MOVES = LS_ST + 8, LS3_XCHG = LS3_MOVES + 64, LS3_POS = LS3_XCHG + 8;   // coop words of commands 4 and 5
+
+// command 5, every warp of the block
+__device__ __forceinline__ void ls3_coop_rewrite(const LsMem &M)
+{
+    const int *x = M.coop + LS3_XCHG;
+    Xchg X;
+    X.r = x[0];
+    X.e[0] = x[1]; X.e[1] = x[2]; X.e[2] = x[3];
+    X.seg[0] = x[4] & 1; X.seg[1] = (x[4] >> 1) & 1;
+    X.rev[0] = x[5] & 1; X.rev[1] = (x[5] >> 1) & 1;
+    const int nth = 32 * M.coop_warps;
+    ls3_rewrite_part(M, X, (int)threadIdx.x, nth, 0);
+    ls_coop_bar(M.coop_warps);
+    ls3_rewrite_part(M, X, (int)threadIdx.x, nth, 1);
+    ls_coop_bar(M.coop_warps);
+}
+
+// rewrites the middle positions of the planned exchange (warp 0)
+__device__ __forceinline__ void ls3_apply(const LsMem &M, const Xchg &X)
+{
+    const int lane = threadIdx.x & 31;
     __syncwarp();
-    for (int w = lane; w < total; w += 32) {
-        const int c = tmp[w];
-        M.tour[lo + w] = c;
-        M.pos[c] = lo + w;
+    if (M.coop && X.e[X.r - 1] - X.e[0] >= LS_COOP_LEN) {
+        if (lane == 0) {
+            int *x = M.coop + LS3_XCHG;
+            M.coop[0] = 5;
+            x[0] = X.r; x[1] = X.e[0]; x[2] = X.e[1]; x[3] = X.r == 3 ? X.e[2] : 0;
+            x[4] = X.seg[0] | (X.r == 3 ? X.seg[1] << 1 : 0);
+            x[5] = X.rev[0] | (X.r == 3 ? X.rev[1] << 1 : 0);
+        }
+        __syncwarp();
+        ls_coop_bar(M.coop_warps);
+        ls3_coop_rewrite(M);
+        return;
     }
+    ls3_rewrite_part(M, X, lane, 32, 0);
+    __syncwarp();
+    ls3_rewrite_part(M, X, lane, 32, 1);
     __syncwarp();
 }
 
@@ -171,9 +220,186 @@ __device__ __forceinline__ Xchg ls3_bcast(const Xchg &X, int src)
     return Y;
 }
 
-// One examination of city a: finds and applies the first admissible move;
-// true if a move was made (its cities' bits cleared).
-__device__ __forceinline__ bool ls3_examine(const DevInst &I, const LsMem &M, int n, int K, int a)
+// the FP64 gain of six terms from FP32 estimates of them: 0 certainly <=
+// LS_GAIN, 2 certainly above, 1 undecided
+__device__ __forceinline__ int ls3_gain_class(float g2, float mag2, float d56, float d61)
+{
+    const float est = __fsub_rn(__fadd_rn(g2, d56), d61);
+    const float tol = __fadd_rn(__fmul_rn(4e-6f, __fadd_rn(mag2, __fadd_rn(d56, d61))), 1e-18f);
+    if (!(est > __fsub_rn((float)LS_GAIN, tol))) return 0;
+    return est > __fadd_rn((float)LS_GAIN, tol) ? 2 : 1;
+}
+
+// What ls3_scan found: st 0 no move; 1 the city's first move, certain; 2 a
+// possible move, undecided in FP32.  c = t1..t4 (r = 2) or t1..t6 (r = 3).
+struct Ls3Move {
+    int st, r, c[6];
+};
+
+// FP32 scan of city a (whole warp, only reads; the same result in every lane)
+__device__ __forceinline__ Ls3Move ls3_scan(const DevInst &I, const LsMem &M, int n, int K, int a)
+{
+    const int lane = threadIdx.x & 31;
+    const float2 *xy = M.xy;
+    const int pa = M.pos[a];
+    const int ts = M.tour[wrap_next(pa, n)], tp = M.tour[wrap_prev(pa, n)];
+    const float ds = ls_d32(xy, ts, a), dp = ls_d32(xy, tp, a);
+    const int nl = lane < K ? I.nbr[(size_t)a * K + lane] : 0;
+    const float dl = lane < K ? I.nbrd32[(size_t)a * K + lane] : __int_as_float(0x7f800000);
+    // t3 candidates of each direction: a prefix of the ascending list
+    const float lim = __fmul_rn(dl, LS_G1_LO);
+    const int Q0 = __popc(__ballot_sync(FULL2, ds > lim)), Q1 = __popc(__ballot_sync(FULL2, dp > lim));
+    const int P = 2 * (Q0 + Q1);
+    Ls3Move F;
+    F.st = 0;
+    F.r = 0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) F.c[k] = 0;
+    for (int base = 0; base < P; base += 32) {
+        const int pi = base + lane;
+        const bool act = pi < P;
+        const int dir = pi >= 2 * Q0 ? 1 : 0, qq = dir ? pi - 2 * Q0 : pi, q = qq >> 1, c4 = qq & 1;
+        const int t3 = __shfl_sync(FULL2, nl, q & 31);
+        const float d23 = __shfl_sync(FULL2, dl, q & 31);
+        const int t1 = dir ? tp : ts, t2 = a;
+        const float d12 = dir ? dp : ds;
+        int st = 0, r = 0, t4 = 0, t5 = 0, t6 = 0;
+        if (act && t3 != t1) {                 // t3 = t1: g1 = 0
+            const int p3 = M.pos[t3];
+            t4 = M.tour[c4 == dir ? wrap_next(p3, n) : wrap_prev(p3, n)];
+            if (!((t3 == t1 && t4 == t2) || (t3 == t2 && t4 == t1))) {
+                const float d34 = ls_d32(xy, t3, t4);
+                const bool g1sure = __fmul_rn(d12, LS_G1_LO) > d23;
+                Xchg X;
+                // t4 = t2 closes to the same tour: its FP64 gain is the rounding of
+                // ((d12 - d23) + d23) - d12, below 1e-10 at these lengths
+                if (c4 == 0 && t4 != t1 && !(t4 == t2 && d12 + d23 < 1e4f)) {
+                    const int cl = ls_gain_class(d12, d23, d34, ls_d32(xy, t4, t1));
+                    if (cl) {
+                        const int c[4] = {t1, t2, t3, t4};
+                        if (ls3_plan<2>(M, n, c, X)) { st = cl == 2 && g1sure ? 1 : 2; r = 2; }
+                    }
+                }
+                const float g1b = __fadd_rn(__fsub_rn(d12, d23), d34), mag1 = __fadd_rn(__fadd_rn(d12, d23), d34);
+                const int32_t *nb4 = I.nbr + (size_t)t4 * K;
+                const float *nd4 = I.nbrd32 + (size_t)t4 * K;
+                for (int k0 = 0; k0 < K && !st; k0 += 4) {
+                    // four t5 at a time, both t6 of each: independent loads
+                    int u5[4], u6[4][2];
+                    float g2[4], mag2[4], d56[4][2], d61[4][2];
+                    bool may[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const bool in = k0 + j < K;
+                        u5[j] = in ? nb4[k0 + j] : t4;
+                        const float d45 = in ? nd4[k0 + j] : __int_as_float(0x7f800000);
+                        g2[j] = __fsub_rn(g1b, d45);
+                        mag2[j] = __fadd_rn(mag1, d45);
+                        may[j] = in && g2[j] > -__fadd_rn(__fmul_rn(4e-6f, mag2[j]), 1e-18f);
+                    }
+                    if (!may[0]) break;                       // the list ascends
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int p5 = M.pos[u5[j]];
+                        u6[j][0] = M.tour[wrap_next(p5, n)];
+                        u6[j][1] = M.tour[wrap_prev(p5, n)];
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int c6 = 0; c6 < 2; ++c6) {
+                            d56[j][c6] = ls_d32(xy, u5[j], u6[j][c6]);
+                            d61[j][c6] = ls_d32(xy, u6[j][c6], t1);
+                        }
+                    unsigned cand = 0u, sure = 0u;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int c6 = 0; c6 < 2; ++c6) {
+                            const int cl = ls3_gain_class(g2[j], mag2[j], d56[j][c6], d61[j][c6]);
+                            // t4 = t2, t5 = t1 adds the edges it removes: gain 0 up to rounding, as above
+                            const bool null = t4 == t2 && u5[j] == t1 && mag2[j] + d56[j][c6] < 1e4f;
+                            const bool ok = may[j] && cl && u5[j] != t3 && u6[j][c6] != t1 && !null;
+                            const bool g2sure = g2[j] > __fadd_rn(__fmul_rn(4e-6f, mag2[j]), 1e-18f);
+                            cand |= (ok ? 1u : 0u) << (2 * j + c6);
+                            sure |= (cl == 2 && g2sure ? 1u : 0u) << (2 * j + c6);
+                        }
+                    while (cand) {                             // rare: is the reconnection one cycle?
+                        const int x = __ffs(cand) - 1;
+                        cand &= cand - 1u;
+                        t5 = nb4[k0 + (x >> 1)];
+                        const int p5 = M.pos[t5];
+                        t6 = M.tour[(x & 1) == 0 ? wrap_next(p5, n) : wrap_prev(p5, n)];
+                        const int c[6] = {t1, t2, t3, t4, t5, t6};
+                        if (ls3_plan<3>(M, n, c, X)) {
+                            st = ((sure >> x) & 1u) && g1sure ? 1 : 2;
+                            r = 3;
+                            break;
+                        }
+                    }
+                    if (!may[3]) break;
+                }
+            }
+        }
+        const unsigned hm = __ballot_sync(FULL2, st != 0);
+        if (hm) {
+            const int src = __ffs(hm) - 1;
+            F.st = __shfl_sync(FULL2, st, src);
+            F.r = __shfl_sync(FULL2, r, src);
+            F.c[0] = __shfl_sync(FULL2, t1, src);
+            F.c[1] = a;
+            F.c[2] = __shfl_sync(FULL2, t3, src);
+            F.c[3] = __shfl_sync(FULL2, t4, src);
+            F.c[4] = __shfl_sync(FULL2, t5, src);
+            F.c[5] = __shfl_sync(FULL2, t6, src);
+            return F;
+        }
+    }
+    return F;
+}
+
+// command 4, every warp of the block: the warp's staged city
+__device__ __forceinline__ void ls3_coop_scan(const DevInst &I, const LsMem &M)
+{
+    const int w = threadIdx.x >> 5;
+    if (w >= M.coop[1]) return;
+    const Ls3Move F = ls3_scan(I, M, I.n, I.ls_k, M.coop[LS_ST + w]);
+    if ((threadIdx.x & 31) == 0) {
+        int *o = M.coop + LS3_MOVES + 8 * w;
+        o[0] = F.st;
+        o[1] = F.r;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[2 + k] = F.c[k];
+    }
+    __syncwarp();
+}
+
+// applies a certain move (warp 0)
+__device__ __forceinline__ void ls3_apply_move(const LsMem &M, int n, const Ls3Move &F)
+{
+    const int lane = threadIdx.x & 31;
+    Xchg X;
+    if (F.r == 2) {
+        const int c[4] = {F.c[0], F.c[1], F.c[2], F.c[3]};
+        ls3_plan<2>(M, n, c, X);
+    } else {
+        ls3_plan<3>(M, n, F.c, X);
+    }
+    ls3_apply(M, X);
+    if (lane < 2 * F.r) {
+        int c = F.c[0];
+#pragma unroll
+        for (int k = 1; k < 6; ++k) c = lane == k ? F.c[k] : c;
+        M.dlb[c] = 0;
+    }
+    __syncwarp();
+}
+
+// One examination of city a in FP64: finds and applies the first admissible
+// move; true if a move was made (its cities' bits cleared).  One t5 per lane
+// (both t6 of it), the first lane with an admissible move wins; the g1 values
+// of all t3 are computed at once, one per lane.
+static __device__ __noinline__ bool ls3_examine(const DevInst &I, const LsMem &M, int n, int K, int a)
 {
     const int lane = threadIdx.x & 31;
     const float2 *xy = M.xy;
@@ -410,6 +636,7 @@ static __device__ __noinline__ void warp_three_opt(const DevInst &I, int32_t *to
     __syncwarp();
     for (int p = lane; p < n; p += 32) M.pos[M.tour[p]] = p;
     __syncwarp();
+    const int W = M.coop ? M.coop_warps : 1;      // cities tested at once (at most LS_WARPS_MAX)
     const long long max_moves = 64LL * n + 1024;
     long long moves = 0;
     int round_moves;
@@ -420,25 +647,72 @@ static __device__ __noinline__ void warp_three_opt(const DevInst &I, int32_t *to
         bool improved = true;
         while (improved && moves < max_moves) {
             improved = false;
-            int p = 0;
-            while (p < n && moves < max_moves) {
-                const int pp = p + lane;
-                const bool clear = pp < n && !M.dlb[M.tour[pp]];
-                const unsigned cm = __ballot_sync(FULL2, clear);
-                if (!cm) { p += 32; continue; }
-                p += __ffs(cm) - 1;
-                const int a = M.tour[p];
-                for (;;) {
-                    const bool moved = ls3_examine(I, M, n, K, a);
-                    if (!moved) break;
+            int p = 0, cur = -1;      // next position of the pass; city to examine again after its move
+            while (moves < max_moves) {
+                // the next cities in order: cur, then the clear ones from position p on
+                // (staged in coop with their positions when there are helpers)
+                int cnt = cur >= 0 ? 1 : 0, city = cur, where = p - 1, q = p;
+                if (W > 1 && cur >= 0 && lane == 0) { M.coop[LS_ST] = cur; M.coop[LS3_POS] = p - 1; }
+                while (cnt < W && q < n) {
+                    const int pp = q + lane;
+                    const int u = pp < n ? M.tour[pp] : 0;
+                    const bool clear = pp < n && u != cur && !M.dlb[u];
+                    const unsigned cm = __ballot_sync(FULL2, clear);
+                    if (W > 1) {
+                        const int d = cnt + __popc(cm & ((1u << lane) - 1u));
+                        if (clear && d < W) { M.coop[LS_ST + d] = u; M.coop[LS3_POS + d] = pp; }
+                        cnt = min(W, cnt + __popc(cm));
+                    } else if (cm) {
+                        where = q + __ffs(cm) - 1;
+                        city = __shfl_sync(FULL2, u, __ffs(cm) - 1);
+                        cnt = 1;
+                    }
+                    q += 32;
+                }
+                __syncwarp();
+                if (W > 1 && lane < cnt) { city = M.coop[LS_ST + lane]; where = M.coop[LS3_POS + lane]; }
+                if (!cnt) break;
+                Ls3Move F;
+                int f = 0;            // the first of them with a possible move
+                if (W > 1 && cnt > 1) {
+                    if (lane == 0) { M.coop[0] = 4; M.coop[1] = cnt; }
+                    __syncwarp();
+                    ls_coop_bar(M.coop_warps);
+                    ls3_coop_scan(I, M);
+                    ls_coop_bar(M.coop_warps);
+                    const unsigned hm = __ballot_sync(FULL2, lane < cnt && M.coop[LS3_MOVES + 8 * (lane & 7)] != 0);
+                    f = hm ? __ffs(hm) - 1 : cnt;
+                    const int *o = M.coop + LS3_MOVES + 8 * (hm ? f : 0);
+                    F.st = hm ? o[0] : 0;
+                    F.r = o[1];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) F.c[k] = o[2 + k];
+                } else {
+                    F = ls3_scan(I, M, n, K, __shfl_sync(FULL2, city, 0));
+                    f = F.st ? 0 : cnt;
+                }
+                if (lane < cnt && lane < f) M.dlb[city] = 1;      // examined, no move
+                __syncwarp();
+                if (!F.st) {          // none of them moves
+                    p = __shfl_sync(FULL2, where, cnt - 1) + 1;
+                    cur = -1;
+                    continue;
+                }
+                const int a = __shfl_sync(FULL2, city, f);
+                p = __shfl_sync(FULL2, where, f) + 1;
+                bool moved = true;
+                if (F.st == 1) ls3_apply_move(M, n, F);
+                else moved = ls3_examine(I, M, n, K, a);
+                if (moved) {
                     improved = true;
                     ++round_moves;
                     ++moves;
-                    if (moves >= max_moves) break;
+                    cur = a;
+                } else {
+                    if (lane == 0) M.dlb[a] = 1;
+                    __syncwarp();
+                    cur = -1;
                 }
-                if (lane == 0) M.dlb[a] = 1;
-                __syncwarp();
-                ++p;
             }
         }
     } while (round_moves > 0 && moves < max_moves);

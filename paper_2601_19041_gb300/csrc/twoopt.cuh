@@ -87,14 +87,18 @@ struct LsMem {
 //     writes what it found, and every warp arrives again; warp 0 takes the
 //     successor move if there is one, else warp 1's (the order of the
 //     sequential search);
+//   4 (3-opt: test up to `warps` cities): warp w tests the w-th staged city
+//     (ls3_scan, threeopt.cuh) and writes what it found; every warp arrives;
+//   5 (3-opt: rewrite the middle of an exchange): every warp copies its share
+//     out, arrives, copies it back in, arrives;
 //   0: the helpers return.
 // Every path through the search ends with command 0.
 constexpr int LS_COOP_LEN = 192;   // reversals of at least this many positions are shared
-// coop words: [0] command (0 exit, 1 reverse, 2 pre-test, 3 examine), [1] i0,
-// item count or city, [2] len; [3..8] warp 1's predecessor move (found, an, b,
+// coop words: [0] command, [1] i0, item count, city or city count, [2] len; [3..8] warp 1's predecessor move (found, an, b,
 // bn, d(a,b) and d(an,bn) as FP32 bits); from LS_ST the staged cities (al,
 // an0, an1, c0, incl, da0, da1; 32 each); from LS_MIN the per-warp minima of
-// two rounds (2 x 8)
+// two rounds (2 x 8); commands 4 and 5 use the words from LS_ST for the staged
+// cities (8), the moves found (8 each) and the exchange (8)
 constexpr int LS_ST = 10, LS_MIN = LS_ST + 7 * 32, LS_COOP_WORDS = LS_MIN + 16;
 constexpr int LS_WARPS_MAX = 8;
 
@@ -225,6 +229,8 @@ __device__ __forceinline__ int ls_pretest_rounds(const DevInst &I, const LsMem &
 }
 
 __device__ __forceinline__ void ls_pred_search(const DevInst &I, const LsMem &M, int a);
+__device__ __forceinline__ void ls3_coop_scan(const DevInst &I, const LsMem &M);
+__device__ __forceinline__ void ls3_coop_rewrite(const LsMem &M);
 
 // the helper warps' side of the protocol above (warps 1 .. coop_warps-1)
 __device__ __forceinline__ void ls_coop_help(const DevInst &I, const LsMem &M)
@@ -241,6 +247,11 @@ __device__ __forceinline__ void ls_coop_help(const DevInst &I, const LsMem &M)
         } else if (cmd == 3) {
             if ((threadIdx.x >> 5) == 1) ls_pred_search(I, M, M.coop[1]);
             ls_coop_bar(M.coop_warps);
+        } else if (cmd == 4) {
+            ls3_coop_scan(I, M);
+            ls_coop_bar(M.coop_warps);
+        } else if (cmd == 5) {
+            ls3_coop_rewrite(M);
         } else {
             break;
         }
