@@ -19,8 +19,8 @@
 //   Gains are FP64, each operation rounded once, in the order written.
 //
 // FP32 scan.  As in the 2-opt, gains are first estimated from FP32 distances
-// (ls_d32, each within 4 units of 2^-24 of the FP64 one): with a band of 4e-6
-// of the terms' sum (six terms and five additions err by less than 6e-7 of
+// (ls_da32, each within 5 units of 2^-24 of the FP64 one): with a band of 4e-6
+// of the terms' sum (six terms and five additions err by less than 6.6e-7 of
 // it) an estimate outside the band decides, and g1 > 0 and g2 > 0 likewise.
 // ls3_scan tests one city: its (direction, t3, t4) pairs with g1 possibly
 // positive are dealt to the lanes, each lane running through its pair's t5
@@ -31,7 +31,7 @@
 // 100 cycles with its use, a distance several hundred): with FP64 alone one
 // search took 47 ms (n = 500, 10-node lists, m = 32, start tour from the ants),
 // and 8 iterations of 32 such instances 469 ms end to end; with the scan and the
-// helper warps they take 41 ms.
+// helper warps they take 30 ms.
 //
 // Helper warps (a block of several warps, see twoopt.cuh) test the next clear
 // cities in tour order at the same time, one per warp: cities before the first
@@ -164,12 +164,10 @@ __device__ __forceinline__ void ls3_rewrite_part(const LsMem &M, const Xchg &X, 
     }
 }
 
-constexpr int LS3_MOVES = LS_ST + 8, LS3_XCHG = LS3_MOVES + 64, LS3_POS = LS3_XCHG + 8;   // coop words of commands 4 and 5
-
-// command 5, every warp of the block
+// command 3, every warp of the block
 __device__ __forceinline__ void ls3_coop_rewrite(const LsMem &M)
 {
-    const int *x = M.coop + LS3_XCHG;
+    const int *x = M.coop + LS_XCHG;
     Xchg X;
     X.r = x[0];
     X.e[0] = x[1]; X.e[1] = x[2]; X.e[2] = x[3];
@@ -189,8 +187,8 @@ __device__ __forceinline__ void ls3_apply(const LsMem &M, const Xchg &X)
     __syncwarp();
     if (M.coop && X.e[X.r - 1] - X.e[0] >= LS_COOP_LEN) {
         if (lane == 0) {
-            int *x = M.coop + LS3_XCHG;
-            M.coop[0] = 5;
+            int *x = M.coop + LS_XCHG;
+            M.coop[0] = 3;
             x[0] = X.r; x[1] = X.e[0]; x[2] = X.e[1]; x[3] = X.r == 3 ? X.e[2] : 0;
             x[4] = X.seg[0] | (X.r == 3 ? X.seg[1] << 1 : 0);
             x[5] = X.rev[0] | (X.r == 3 ? X.rev[1] << 1 : 0);
@@ -230,27 +228,22 @@ __device__ __forceinline__ int ls3_gain_class(float g2, float mag2, float d56, f
     return est > __fadd_rn((float)LS_GAIN, tol) ? 2 : 1;
 }
 
-// What ls3_scan found: st 0 no move; 1 the city's first move, certain; 2 a
-// possible move, undecided in FP32.  c = t1..t4 (r = 2) or t1..t6 (r = 3).
-struct Ls3Move {
-    int st, r, c[6];
-};
-
 // FP32 scan of city a (whole warp, only reads; the same result in every lane)
-__device__ __forceinline__ Ls3Move ls3_scan(const DevInst &I, const LsMem &M, int n, int K, int a)
+__device__ __forceinline__ LsMove ls3_scan(const LsMem &M, int n, int K, int a)
 {
     const int lane = threadIdx.x & 31;
     const float2 *xy = M.xy;
     const int pa = M.pos[a];
     const int ts = M.tour[wrap_next(pa, n)], tp = M.tour[wrap_prev(pa, n)];
-    const float ds = ls_d32(xy, ts, a), dp = ls_d32(xy, tp, a);
-    const int nl = lane < K ? I.nbr[(size_t)a * K + lane] : 0;
-    const float dl = lane < K ? I.nbrd32[(size_t)a * K + lane] : __int_as_float(0x7f800000);
+    const float2 xa = xy[a], xs = xy[ts], xp = xy[tp];
+    const float ds = ls_da32(xs, xa), dp = ls_da32(xp, xa);
+    const int nl = lane < K ? M.nbr[(size_t)a * K + lane] : 0;
+    const float dl = lane < K ? M.nbrd32[(size_t)a * K + lane] : __int_as_float(0x7f800000);
     // t3 candidates of each direction: a prefix of the ascending list
     const float lim = __fmul_rn(dl, LS_G1_LO);
     const int Q0 = __popc(__ballot_sync(FULL2, ds > lim)), Q1 = __popc(__ballot_sync(FULL2, dp > lim));
     const int P = 2 * (Q0 + Q1);
-    Ls3Move F;
+    LsMove F;
     F.st = 0;
     F.r = 0;
 #pragma unroll
@@ -268,21 +261,22 @@ __device__ __forceinline__ Ls3Move ls3_scan(const DevInst &I, const LsMem &M, in
             const int p3 = M.pos[t3];
             t4 = M.tour[c4 == dir ? wrap_next(p3, n) : wrap_prev(p3, n)];
             if (!((t3 == t1 && t4 == t2) || (t3 == t2 && t4 == t1))) {
-                const float d34 = ls_d32(xy, t3, t4);
+                const float2 x1 = dir ? xp : xs, x4 = xy[t4];
+                const float d34 = ls_da32(xy[t3], x4);
                 const bool g1sure = __fmul_rn(d12, LS_G1_LO) > d23;
                 Xchg X;
                 // t4 = t2 closes to the same tour: its FP64 gain is the rounding of
                 // ((d12 - d23) + d23) - d12, below 1e-10 at these lengths
                 if (c4 == 0 && t4 != t1 && !(t4 == t2 && d12 + d23 < 1e4f)) {
-                    const int cl = ls_gain_class(d12, d23, d34, ls_d32(xy, t4, t1));
+                    const int cl = ls_gain_class(d12, d23, d34, ls_da32(x4, x1));
                     if (cl) {
                         const int c[4] = {t1, t2, t3, t4};
                         if (ls3_plan<2>(M, n, c, X)) { st = cl == 2 && g1sure ? 1 : 2; r = 2; }
                     }
                 }
                 const float g1b = __fadd_rn(__fsub_rn(d12, d23), d34), mag1 = __fadd_rn(__fadd_rn(d12, d23), d34);
-                const int32_t *nb4 = I.nbr + (size_t)t4 * K;
-                const float *nd4 = I.nbrd32 + (size_t)t4 * K;
+                const int32_t *nb4 = M.nbr + (size_t)t4 * K;
+                const float *nd4 = M.nbrd32 + (size_t)t4 * K;
                 for (int k0 = 0; k0 < K && !st; k0 += 4) {
                     // four t5 at a time, both t6 of each: independent loads
                     int u5[4], u6[4][2];
@@ -305,12 +299,15 @@ __device__ __forceinline__ Ls3Move ls3_scan(const DevInst &I, const LsMem &M, in
                         u6[j][1] = M.tour[wrap_prev(p5, n)];
                     }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 x5 = xy[u5[j]];
 #pragma unroll
                         for (int c6 = 0; c6 < 2; ++c6) {
-                            d56[j][c6] = ls_d32(xy, u5[j], u6[j][c6]);
-                            d61[j][c6] = ls_d32(xy, u6[j][c6], t1);
+                            const float2 x6 = xy[u6[j][c6]];
+                            d56[j][c6] = ls_da32(x5, x6);
+                            d61[j][c6] = ls_da32(x6, x1);
                         }
+                    }
                     unsigned cand = 0u, sure = 0u;
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
@@ -358,24 +355,8 @@ __device__ __forceinline__ Ls3Move ls3_scan(const DevInst &I, const LsMem &M, in
     return F;
 }
 
-// command 4, every warp of the block: the warp's staged city
-__device__ __forceinline__ void ls3_coop_scan(const DevInst &I, const LsMem &M)
-{
-    const int w = threadIdx.x >> 5;
-    if (w >= M.coop[1]) return;
-    const Ls3Move F = ls3_scan(I, M, I.n, I.ls_k, M.coop[LS_ST + w]);
-    if ((threadIdx.x & 31) == 0) {
-        int *o = M.coop + LS3_MOVES + 8 * w;
-        o[0] = F.st;
-        o[1] = F.r;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) o[2 + k] = F.c[k];
-    }
-    __syncwarp();
-}
-
 // applies a certain move (warp 0)
-__device__ __forceinline__ void ls3_apply_move(const LsMem &M, int n, const Ls3Move &F)
+__device__ __forceinline__ void ls3_apply_move(const LsMem &M, int n, const LsMove &F)
 {
     const int lane = threadIdx.x & 31;
     Xchg X;
@@ -636,89 +617,71 @@ static __device__ __noinline__ void warp_three_opt(const DevInst &I, int32_t *to
     __syncwarp();
     for (int p = lane; p < n; p += 32) M.pos[M.tour[p]] = p;
     __syncwarp();
-    const int W = M.coop ? M.coop_warps : 1;      // cities tested at once (at most LS_WARPS_MAX)
-    const long long max_moves = 64LL * n + 1024;
-    long long moves = 0;
-    int round_moves;
-    do {
-        round_moves = 0;
-        for (int p = lane; p < n; p += 32) M.dlb[p] = 0;
-        __syncwarp();
-        bool improved = true;
-        while (improved && moves < max_moves) {
-            improved = false;
-            int p = 0, cur = -1;      // next position of the pass; city to examine again after its move
-            while (moves < max_moves) {
-                // the next cities in order: cur, then the clear ones from position p on
-                // (staged in coop with their positions when there are helpers)
-                int cnt = cur >= 0 ? 1 : 0, city = cur, where = p - 1, q = p;
-                if (W > 1 && cur >= 0 && lane == 0) { M.coop[LS_ST] = cur; M.coop[LS3_POS] = p - 1; }
-                while (cnt < W && q < n) {
-                    const int pp = q + lane;
-                    const int u = pp < n ? M.tour[pp] : 0;
-                    const bool clear = pp < n && u != cur && !M.dlb[u];
-                    const unsigned cm = __ballot_sync(FULL2, clear);
-                    if (W > 1) {
-                        const int d = cnt + __popc(cm & ((1u << lane) - 1u));
-                        if (clear && d < W) { M.coop[LS_ST + d] = u; M.coop[LS3_POS + d] = pp; }
-                        cnt = min(W, cnt + __popc(cm));
-                    } else if (cm) {
-                        where = q + __ffs(cm) - 1;
-                        city = __shfl_sync(FULL2, u, __ffs(cm) - 1);
-                        cnt = 1;
-                    }
-                    q += 32;
-                }
-                __syncwarp();
-                if (W > 1 && lane < cnt) { city = M.coop[LS_ST + lane]; where = M.coop[LS3_POS + lane]; }
-                if (!cnt) break;
-                Ls3Move F;
-                int f = 0;            // the first of them with a possible move
-                if (W > 1 && cnt > 1) {
-                    if (lane == 0) { M.coop[0] = 4; M.coop[1] = cnt; }
-                    __syncwarp();
-                    ls_coop_bar(M.coop_warps);
-                    ls3_coop_scan(I, M);
-                    ls_coop_bar(M.coop_warps);
-                    const unsigned hm = __ballot_sync(FULL2, lane < cnt && M.coop[LS3_MOVES + 8 * (lane & 7)] != 0);
-                    f = hm ? __ffs(hm) - 1 : cnt;
-                    const int *o = M.coop + LS3_MOVES + 8 * (hm ? f : 0);
-                    F.st = hm ? o[0] : 0;
-                    F.r = o[1];
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) F.c[k] = o[2 + k];
-                } else {
-                    F = ls3_scan(I, M, n, K, __shfl_sync(FULL2, city, 0));
-                    f = F.st ? 0 : cnt;
-                }
-                if (lane < cnt && lane < f) M.dlb[city] = 1;      // examined, no move
-                __syncwarp();
-                if (!F.st) {          // none of them moves
-                    p = __shfl_sync(FULL2, where, cnt - 1) + 1;
-                    cur = -1;
-                    continue;
-                }
-                const int a = __shfl_sync(FULL2, city, f);
-                p = __shfl_sync(FULL2, where, f) + 1;
-                bool moved = true;
-                if (F.st == 1) ls3_apply_move(M, n, F);
-                else moved = ls3_examine(I, M, n, K, a);
-                if (moved) {
-                    improved = true;
-                    ++round_moves;
-                    ++moves;
-                    cur = a;
-                } else {
-                    if (lane == 0) M.dlb[a] = 1;
-                    __syncwarp();
-                    cur = -1;
-                }
-            }
-        }
-    } while (round_moves > 0 && moves < max_moves);
+    ls_rounds_ahead<true, false>(M, n, K, 1, [&](int a) { return ls3_scan(M, n, K, a); },
+                    [&](const LsMove &F) { ls3_apply_move(M, n, F); }, [&](int a) { return ls3_examine(I, M, n, K, a); });
     if (M.tour != tour)
         for (int p = lane; p < n; p += 32) tour[p] = M.tour[p];
     __syncwarp();
+}
+
+// The search of a symmetric instance by a whole block (every thread calls it):
+// `tour` improved in place, warp 0 in control, the other warps helping.
+__device__ __forceinline__ void block_search(const DevInst &I, int32_t *tour, const LsMem &M)
+{
+    const int n = I.n, K = I.ls_k;
+    if (M.tour != tour)
+        for (int p = threadIdx.x; p < n; p += blockDim.x) M.tour[p] = tour[p];
+    __syncthreads();
+    for (int p = threadIdx.x; p < n; p += blockDim.x) M.pos[M.tour[p]] = p;
+    __syncthreads();
+    if (threadIdx.x >= 32) {
+        ls_coop_help(I, M);
+    } else {
+        if (I.local_search >= 3)
+            ls_rounds_ahead<true, true>(M, n, K, M.coop_warps, [&](int a) { return ls3_scan(M, n, K, a); },
+                                  [&](const LsMove &F) { ls3_apply_move(M, n, F); },
+                                  [&](int a) { return ls3_examine(I, M, n, K, a); });
+        else
+            ls_rounds_ahead<false, true>(M, n, K, M.coop_warps, [&](int a) { return ls2_scan(M, n, K, a); },
+                                   [&](const LsMove &F) { ls2_apply(M, n, F); },
+                                   [&](int a) {
+                                       const LsMove F = ls2_exact(I, M, n, K, a);
+                                       if (F.st) ls2_apply(M, n, F);
+                                       return F.st != 0;
+                                   });
+        ls_coop_end(M);
+    }
+    __syncthreads();
+    if (M.tour != tour)
+        for (int p = threadIdx.x; p < n; p += blockDim.x) tour[p] = M.tour[p];
+    __syncthreads();
+}
+
+// The local search of T_NN and T_ib, a block of several warps per tour, with
+// its arrays in the block's shared memory where they fit.  The case that all
+// of them fit has code of its own, in which the compiler knows their address
+// space: through pointers that may be either, an n = 10000 search took 11.3 ms
+// instead of 8.7.
+__device__ __forceinline__ void block_local_search(const DevInst &I, int32_t *tour, unsigned char *sm, size_t smem_bytes,
+                                                   int *coop)
+{
+    const int warps = (int)(blockDim.x >> 5);
+    if (I.kind == 1) {                 // directed: one warp, no helpers
+        if (threadIdx.x < 32) warp_two_opt_directed(I, tour, ls_shared(I, tour, sm, smem_bytes, ls_global(I, tour)));
+        __syncthreads();
+    } else if (ls_smem_full(I.n) <= smem_bytes) {
+        LsMem M = ls_shared_full(I, sm);
+        float2 *sxy = reinterpret_cast<float2 *>(sm + ls_xy_offset(I.n));
+        for (int p = threadIdx.x; p < I.n; p += blockDim.x) sxy[p] = reinterpret_cast<const float2 *>(I.xy)[p];
+        M.coop = coop;
+        M.coop_warps = warps;
+        block_search(I, tour, M);
+    } else {
+        LsMem M = ls_shared(I, tour, sm, smem_bytes, ls_global(I, tour), false);
+        M.coop = coop;
+        M.coop_warps = warps;
+        block_search(I, tour, M);
+    }
 }
 
 }  // namespace hac

@@ -1,13 +1,13 @@
-// Local-search kernels (one warp per tour, its arrays in shared memory when
-// they fit): 2-opt (local_search 1 and 2; twoopt.cuh, or the directed 2-opt of
+// Local-search kernels (a block or a warp per tour, its arrays in shared memory
+// when they fit): 2-opt (local_search 1 and 2; twoopt.cuh, or the directed 2-opt of
 // threeopt.cuh for the ATSP) or 3-opt (3 and 4, threeopt.cuh).
 #include "threeopt.cuh"
 
 namespace hac {
 
-// One block of LS_WARPS warps per instance: warp 0 runs the search, the other
-// warps help with its long segment reversals and wide pre-tests (twoopt.cuh,
-// 2-opt of symmetric instances) and are released when it ends.
+// One block of LS_WARPS warps per instance: warp 0 controls the search, the
+// other warps examine the cities after its own and share its long reversals and
+// rewrites (twoopt.cuh; symmetric instances) and are released when it ends.
 constexpr int LS_WARPS = 8;   // at most LS_WARPS_MAX
 
 __global__ void k_two_opt_nn(const DevInst *insts, unsigned smem_bytes)
@@ -16,13 +16,8 @@ __global__ void k_two_opt_nn(const DevInst *insts, unsigned smem_bytes)
     __shared__ int coop[LS_COOP_WORDS];
     const DevInst &I = insts[blockIdx.x];
     if (!I.local_search) return;   // the same for the whole block
-    const bool w0 = threadIdx.x < 32;
-    LsMem M = ls_shared(I, I.nn_tour, ls_sm, smem_bytes, ls_global(I, I.nn_tour), w0);
-    if (blockDim.x > 32) { M.coop = coop; M.coop_warps = (int)(blockDim.x >> 5); }
-    if (!w0) { ls_coop_help(I, M); return; }
-    if (I.local_search >= 3) warp_three_opt(I, I.nn_tour, M);
-    else warp_two_opt_any(I, I.nn_tour, M);
-    ls_coop_end(M);
+    block_local_search(I, I.nn_tour, ls_sm, smem_bytes, coop);
+    if (threadIdx.x >= 32) return;
     const double L = warp_tour_length(I, I.nn_tour);
     if (threadIdx.x == 0) I.st->L_nn = L;
 }
@@ -33,13 +28,8 @@ __global__ void k_two_opt_ib(const DevInst *insts, unsigned smem_bytes)
     __shared__ int coop[LS_COOP_WORDS];
     const DevInst &I = insts[blockIdx.x];
     if ((I.local_search != 1 && I.local_search != 3) || !I.st->active) return;   // the same for the whole block
-    const bool w0 = threadIdx.x < 32;
-    LsMem M = ls_shared(I, I.ib_tour, ls_sm, smem_bytes, ls_global(I, I.ib_tour), w0);
-    if (blockDim.x > 32) { M.coop = coop; M.coop_warps = (int)(blockDim.x >> 5); }
-    if (!w0) { ls_coop_help(I, M); return; }
-    if (I.local_search == 3) warp_three_opt(I, I.ib_tour, M);
-    else warp_two_opt_any(I, I.ib_tour, M);
-    ls_coop_end(M);
+    block_local_search(I, I.ib_tour, ls_sm, smem_bytes, coop);
+    if (threadIdx.x >= 32) return;
     const double L = warp_tour_length(I, I.ib_tour);
     if (threadIdx.x == 0) I.st->L_ib = L;
 }

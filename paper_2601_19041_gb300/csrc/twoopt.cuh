@@ -30,15 +30,27 @@
 // side.  The moves taken are therefore exactly those of the plain FP64 search;
 // the FP32 edge lengths stored for the new edges are FP32 estimates too.
 //
-// Parallelism inside the sequential search: when more than LS_FEW of the
-// next 32 tour positions hold cities whose bit is clear, a pass tests them at
-// once with the FP32 test only, their candidate moves spread over the lanes;
-// the cities before the first one that might move have no move and get their
-// bit at once (as they would one by one, since examining a city without a move
-// changes nothing else).  A city that might move, or the first clear one when
-// few are clear, is examined by the whole warp, one neighbour per lane (FP32
-// classes, then FP64 when the first candidate is undecided).  Segment
-// reversals swap element pairs across lanes.
+// Parallelism inside the sequential search, on one warp (every ant's tour;
+// the cluster kernel): when more than LS_FEW of the next 32 tour positions
+// hold cities whose bit is clear, a pass tests them at once with the FP32 test
+// only, their candidate moves spread over the lanes; the cities before the
+// first one that might move have no move and get their bit at once (as they
+// would one by one, since examining a city without a move changes nothing
+// else).  A city that might move, or the first clear one when few are clear, is
+// examined by the whole warp, one neighbour per lane (FP32 classes, then FP64
+// when the first candidate is undecided).  Segment reversals swap element
+// pairs across lanes.
+//
+// On a block of several warps (T_NN and T_ib in kernels of their own): every
+// warp examines one city (ls2_scan: a neighbour per lane, both directions), the
+// next clear cities in tour order at once, so that one round of the block finds
+// the first city with a move and, unless FP32 leaves it undecided, the move
+// itself; all warps share long reversals.  Moves are dense (4200 moves in 7300
+// rounds per search of an n = 10000 iteration-best tour), so the search is a
+// chain of rounds (740 cycles to find the next clear cities, 1150 to examine
+// them) and moves (760), and its latency is what counts: testing 32 cities' moves
+// on all warps and then examining the first candidate took 18.4 ms per search,
+// this takes 8.2 ms.
 #pragma once
 
 #include "lengths.cuh"
@@ -66,41 +78,31 @@ struct LsMem {
     uint8_t *dlb;       // don't-look bit by city
     float *el;          // el[p] ~ d(tour[p], tour[p+1 mod n]), FP32
     const float2 *xy;   // coordinates
+    const int32_t *nbr = nullptr;     // neighbour lists and their FP32 distances, copied here because a
+    const float *nbrd32 = nullptr;    // pointer read through the instance is read again after every store
     int *coop = nullptr;   // shared command words of the helper warps (null: warp 0 alone)
     int coop_warps = 1;    // warps of the block (warp 0 searches, the others help)
 };
 
-// Helper warps.  The search is sequential and runs in warp 0; in a block of
-// several warps the others wait at named barrier 1 and take their share of
-// each long segment reversal (its element pairs are independent, so the
-// result does not depend on who swaps which pair) and of each wide FP32
-// pre-test of 32 positions (ls_first_may_move, more than 32 work items).
+// Helper warps.  The search is sequential and its control runs in warp 0; in
+// a block of several warps the others wait at named barrier 1 and examine
+// cities and take their share of each long segment reversal (its element pairs
+// are independent, so the result does not depend on who swaps which pair).
 // Protocol: warp 0 writes a command to coop and every warp arrives at the
 // barrier; then
 //   1 (reverse i0 .. i0+len-1): every warp swaps its pairs, arrives again;
-//   2 (pre-test of the staged cities): the block deals the items 32 * warps
-//     at a time, each round ending at the barrier after the per-warp minima
-//     are written; every thread reads the same minima, so all leave after
-//     the same round (the first with a possible move);
-//   3 (examine city a): warp 1 searches a's predecessor direction while
-//     warp 0 searches the successor direction (both only read the tour),
-//     writes what it found, and every warp arrives again; warp 0 takes the
-//     successor move if there is one, else warp 1's (the order of the
-//     sequential search);
-//   4 (3-opt: test up to `warps` cities): warp w tests the w-th staged city
-//     (ls3_scan, threeopt.cuh) and writes what it found; every warp arrives;
-//   5 (3-opt: rewrite the middle of an exchange): every warp copies its share
+//   2 (examine up to `warps` cities): warp w examines the w-th staged city and
+//     writes what it found; every warp arrives again;
+//   3 (3-opt: rewrite the middle of an exchange): every warp copies its share
 //     out, arrives, copies it back in, arrives;
 //   0: the helpers return.
 // Every path through the search ends with command 0.
 constexpr int LS_COOP_LEN = 192;   // reversals of at least this many positions are shared
-// coop words: [0] command, [1] i0, item count, city or city count, [2] len; [3..8] warp 1's predecessor move (found, an, b,
-// bn, d(a,b) and d(an,bn) as FP32 bits); from LS_ST the staged cities (al,
-// an0, an1, c0, incl, da0, da1; 32 each); from LS_MIN the per-warp minima of
-// two rounds (2 x 8); commands 4 and 5 use the words from LS_ST for the staged
-// cities (8), the moves found (8 each) and the exchange (8)
-constexpr int LS_ST = 10, LS_MIN = LS_ST + 7 * 32, LS_COOP_WORDS = LS_MIN + 16;
 constexpr int LS_WARPS_MAX = 8;
+// coop words: [0] command, [1] i0 or city count, [2] len; the staged cities and
+// their positions; the moves found (8 words each); the exchange (8)
+constexpr int LS_ST = 4, LS_POS = LS_ST + LS_WARPS_MAX + 1, LS_MOVES = LS_POS + LS_WARPS_MAX + 1,
+              LS_XCHG = LS_MOVES + 8 * LS_WARPS_MAX, LS_COOP_WORDS = LS_XCHG + 8;
 
 __device__ __forceinline__ void ls_coop_bar(int warps)
 {
@@ -134,7 +136,8 @@ __device__ __forceinline__ bool ls_may_improve(float da, float dab, float dbb, f
 // the element swaps of reversing positions i0 .. i0+len-1 (mod n) that fall to
 // thread `tid` of `nth`: tour/pos pairs and the inner edge lengths; the pairs
 // of different t are disjoint, so each thread loads two pairs before it
-// stores them
+// stores them (EL false: the edge lengths are not kept)
+template <bool EL>
 __device__ __forceinline__ void ls_reverse_part(const LsMem &M, int n, int i0, int len, int tid, int nth)
 {
     const int h = len / 2;
@@ -159,7 +162,7 @@ __device__ __forceinline__ void ls_reverse_part(const LsMem &M, int n, int i0, i
             M.pos[u1] = q1;
         }
     }
-    const int he = (len - 1) / 2;
+    const int he = EL ? (len - 1) / 2 : 0;
     for (int t = tid; t < he; t += 2 * nth) {
         const bool two = t + nth < he;
         int p0 = i0 + t, q0 = i0 + len - 2 - t;
@@ -185,77 +188,263 @@ __device__ __forceinline__ void ls_reverse_part(const LsMem &M, int n, int i0, i
 __device__ __forceinline__ bool ls_item_may_improve(const DevInst &I, const LsMem &M, int n, int K, int a, int dir,
                                                    int q, int an, float da)
 {
-    const int b = I.nbr[(size_t)a * K + q];
-    const float dab = I.nbrd32[(size_t)a * K + q];
+    const int b = M.nbr[(size_t)a * K + q];
+    const float dab = M.nbrd32[(size_t)a * K + q];
     const int pb = M.pos[b];
     const int pe = dir == 0 ? pb : wrap_prev(pb, n);     // the edge (b, dir b)
     const int bn = M.tour[dir == 0 ? wrap_next(pb, n) : pe];
     return b != an && bn != a && ls_may_improve(da, dab, M.el[pe], ls_d32(M.xy, an, bn));
 }
 
-// The block's side of a shared pre-test (every thread of the block): items
-// t = tid, tid + 32*warps, ... of the staged cities, in rounds; the first
-// round with a possible move gives the answer (the smallest staged lane that
-// owns one), as in the warp's own loop.  All threads return the same value.
-__device__ __forceinline__ int ls_pretest_rounds(const DevInst &I, const LsMem &M, int n, int K, int total)
-{
-    const int *st = M.coop + LS_ST;
-    const int *s_al = st, *s_an0 = st + 32, *s_an1 = st + 64, *s_c0 = st + 96, *s_incl = st + 128;
-    const float *s_da0 = reinterpret_cast<const float *>(st + 160), *s_da1 = reinterpret_cast<const float *>(st + 192);
-    int *mins = M.coop + LS_MIN;
-    const int tid = (int)threadIdx.x, nth = 32 * M.coop_warps, w = tid >> 5;
-    for (int base = 0, r = 0; base < total; base += nth, ++r) {
-        const int t = base + tid;
-        int c = 0;
-        bool hit = false;
-        if (t < total) {
-#pragma unroll
-            for (int s2 = 16; s2 >= 1; s2 >>= 1)
-                if (s_incl[c + s2 - 1] <= t) c += s2;
-            const int j = t - (c ? s_incl[c - 1] : 0);
-            const int cc0 = s_c0[c];
-            const int dir = j < cc0 ? 0 : 1;
-            hit = ls_item_may_improve(I, M, n, K, s_al[c], dir, dir == 0 ? j : j - cc0,
-                                      dir == 0 ? s_an0[c] : s_an1[c], dir == 0 ? s_da0[c] : s_da1[c]);
-        }
-        const unsigned wmin = __reduce_min_sync(FULL2, hit ? (unsigned)c : 32u);
-        if ((tid & 31) == 0) mins[(r & 1) * 8 + w] = (int)wmin;
-        ls_coop_bar(M.coop_warps);
-        int first = 32;
-        for (int q = 0; q < M.coop_warps; ++q) first = min(first, mins[(r & 1) * 8 + q]);
-        if (first < 32) return first;
-    }
-    return 32;
-}
+// What the examination of a city in FP32 found: st 0 no move; 1 the city's
+// first move, certain; 2 a possible move, undecided.  2-opt: r is the direction
+// (0 successor) and c = a, dir a, b, dir b; 3-opt: c = t1..t4 (r = 2) or t1..t6
+// (r = 3).
+struct LsMove {
+    int st, r, c[6];
+};
 
-__device__ __forceinline__ void ls_pred_search(const DevInst &I, const LsMem &M, int a);
-__device__ __forceinline__ void ls3_coop_scan(const DevInst &I, const LsMem &M);
+__device__ __forceinline__ LsMove ls3_scan(const LsMem &M, int n, int K, int a);
 __device__ __forceinline__ void ls3_coop_rewrite(const LsMem &M);
 
-// the helper warps' side of the protocol above (warps 1 .. coop_warps-1)
-__device__ __forceinline__ void ls_coop_help(const DevInst &I, const LsMem &M)
+// FP32 distance with the approximate square root (error at most 2^-23 of it):
+// within 5 units of 2^-24, far inside the 4e-6 bands
+__device__ __forceinline__ float ls_da32(float2 p, float2 q)
 {
-    const int n = I.n, nth = 32 * M.coop_warps;
+    const float dx = __fsub_rn(q.x, p.x), dy = __fsub_rn(q.y, p.y);
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy))));
+    return r;
+}
+
+// One city's 2-opt moves in FP32 (whole warp, only reads, the same result in
+// every lane): a neighbour per lane, both directions.
+__device__ __forceinline__ LsMove ls2_scan(const LsMem &M, int n, int K, int a)
+{
+    const int lane = threadIdx.x & 31;
+    const int b = lane < K ? M.nbr[(size_t)a * K + lane] : a;
+    const float nd = lane < K ? M.nbrd32[(size_t)a * K + lane] : __int_as_float(0x7f800000);
+    const int pa = M.pos[a];
+    const int an0 = M.tour[wrap_next(pa, n)], an1 = M.tour[wrap_prev(pa, n)];
+    const float2 xa = M.xy[a], x0 = M.xy[an0], x1 = M.xy[an1];
+    const float da0 = ls_da32(xa, x0), da1 = ls_da32(xa, x1);
+    const float lim = __fmul_rn(nd, LS_G1_LO);
+    const int pb = M.pos[b];
+    const int bn0 = M.tour[wrap_next(pb, n)], bn1 = M.tour[wrap_prev(pb, n)];
+    const float2 xb = M.xy[b], y0 = M.xy[bn0], y1 = M.xy[bn1];
+    const int g0 = ls_gain_class(da0, nd, ls_da32(xb, y0), ls_da32(x0, y0));
+    const int g1 = ls_gain_class(da1, nd, ls_da32(xb, y1), ls_da32(x1, y1));
+    const bool c0 = (da0 > lim) & (g0 != 0) & (b != an0) & (bn0 != a);
+    const bool c1 = (da1 > lim) & (g1 != 0) & (b != an1) & (bn1 != a);
+    const unsigned m0 = __ballot_sync(FULL2, c0), m1 = __ballot_sync(FULL2, c1);
+    LsMove F;
+    F.st = 0;
+    F.r = m0 ? 0 : 1;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) F.c[k] = a;
+    if (!(m0 | m1)) return F;
+    const int src = __ffs(m0 ? m0 : m1) - 1;
+    const bool sure = m0 ? (g0 == 2) & (__fmul_rn(da0, LS_G1_LO) > nd) : (g1 == 2) & (__fmul_rn(da1, LS_G1_LO) > nd);
+    F.st = __shfl_sync(FULL2, sure ? 1 : 2, src);
+    F.c[1] = m0 ? an0 : an1;
+    F.c[2] = __shfl_sync(FULL2, b, src);
+    F.c[3] = __shfl_sync(FULL2, m0 ? bn0 : bn1, src);
+    return F;
+}
+
+// the same city in FP64, when FP32 left its first candidate undecided: the
+// first improving move in order (st 0 or 1)
+static __device__ __noinline__ LsMove ls2_exact(const DevInst &I, const LsMem &M, int n, int K, int a)
+{
+    const int lane = threadIdx.x & 31;
+    const int b = lane < K ? I.nbr[(size_t)a * K + lane] : a;
+    const double nd = lane < K ? I.nbrd[(size_t)a * K + lane] : 0.0;
+    const int pa = M.pos[a], pb = M.pos[b];
+    LsMove F;
+    F.st = 0;
+    F.r = 0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) F.c[k] = a;
+    for (int dir = 0; dir < 2 && !F.st; ++dir) {
+        const int an = M.tour[dir == 0 ? wrap_next(pa, n) : wrap_prev(pa, n)];
+        const int bn = M.tour[dir == 0 ? wrap_next(pb, n) : wrap_prev(pb, n)];
+        bool ok = false;
+        if (lane < K && b != an && bn != a) {
+            const double g1 = __dsub_rn(dist64(I, a, an), nd);
+            if (g1 > 0.0) ok = __dsub_rn(__dadd_rn(g1, dist64(I, b, bn)), dist64(I, an, bn)) > LS_GAIN;
+        }
+        const unsigned m = __ballot_sync(FULL2, ok);
+        if (!m) continue;
+        const int src = __ffs(m) - 1;
+        F.st = 1;
+        F.r = dir;
+        F.c[1] = an;
+        F.c[2] = __shfl_sync(FULL2, b, src);
+        F.c[3] = __shfl_sync(FULL2, bn, src);
+    }
+    return F;
+}
+
+// command 2, every warp of the block: the warp's staged city
+__device__ __forceinline__ void ls_coop_scan(const LsMem &M, int n, int K, bool three)
+{
+    const int w = threadIdx.x >> 5;
+    if (w >= M.coop[1]) return;
+    const int a = M.coop[LS_ST + w];
+    const LsMove F = three ? ls3_scan(M, n, K, a) : ls2_scan(M, n, K, a);
+    if ((threadIdx.x & 31) == 0) {
+        int *o = M.coop + LS_MOVES + 8 * w;
+        o[0] = F.st;
+        o[1] = F.r;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[2 + k] = F.c[k];
+    }
+    __syncwarp();
+}
+
+// the helper warps' side of the protocol above (warps 1 .. coop_warps-1)
+__device__ __forceinline__ void ls_coop_help(const DevInst &I, const LsMem &Mref)
+{
+    const LsMem M = Mref;
+    const int n = I.n, K = I.ls_k, nth = 32 * M.coop_warps;
+    const bool three = I.local_search >= 3;
     for (;;) {
         ls_coop_bar(M.coop_warps);
         const int cmd = M.coop[0];
         if (cmd == 1) {
-            ls_reverse_part(M, n, M.coop[1], M.coop[2], (int)threadIdx.x, nth);
+            ls_reverse_part<false>(M, n, M.coop[1], M.coop[2], (int)threadIdx.x, nth);
             ls_coop_bar(M.coop_warps);
         } else if (cmd == 2) {
-            ls_pretest_rounds(I, M, n, I.ls_k, M.coop[1]);
+            ls_coop_scan(M, n, K, three);
+            ls_coop_bar(M.coop_warps);
         } else if (cmd == 3) {
-            if ((threadIdx.x >> 5) == 1) ls_pred_search(I, M, M.coop[1]);
-            ls_coop_bar(M.coop_warps);
-        } else if (cmd == 4) {
-            ls3_coop_scan(I, M);
-            ls_coop_bar(M.coop_warps);
-        } else if (cmd == 5) {
             ls3_coop_rewrite(M);
         } else {
             break;
         }
     }
+}
+
+template <int V>
+struct LsInt {
+    static constexpr int value = V;
+};
+
+// The passes and rounds of a search with don't-look bits, its cities examined
+// W at a time by the block's warps (AHEAD), or one at a time by this warp alone.  Cities
+// without a move are examined in any order with the same outcome, so the next
+// W clear cities in tour order are examined at once and the first with a move
+// is taken; the others are examined again after it.
+//   scan(a)  the examination of one city; exact(a, F) decides an undecided one:
+//   it makes the move and returns true, or returns false; apply(F) makes a
+//   certain one.  Both clear the bits of the move's cities.
+template <bool THREE, bool AHEAD, typename Scan, typename Apply, typename Exact>
+__device__ __forceinline__ void ls_rounds_ahead(const LsMem &M, int n, int K, int W, Scan &&scan, Apply &&apply,
+                                                Exact &&exact)
+{
+    const int lane = threadIdx.x & 31;
+    const long long max_moves = 64LL * n + 1024;
+    long long moves = 0;
+    int round_moves;
+    do {
+        round_moves = 0;
+        for (int p = lane; p < n; p += 32) M.dlb[p] = 0;
+        __syncwarp();
+        bool improved = true;
+        while (improved && moves < max_moves) {
+            improved = false;
+            int p = 0, cur = -1;      // next position of the pass; city to examine again after its move
+            while (moves < max_moves) {
+                // the next cities in order: cur, then the clear ones from position p on
+                int cnt = cur >= 0 ? 1 : 0, city = cur, where = p - 1, q = p;
+                if constexpr (AHEAD) {
+                    // staged in coop with their positions: 64 positions first (cities are
+                    // dense early in a search), then 256 at a time, the loads of a group
+                    // in flight together; the slot past the last takes what is not wanted
+                    if (cur >= 0 && lane == 0) { M.coop[LS_ST] = cur; M.coop[LS_POS] = p - 1; }
+                    auto gather = [&](auto windows) {
+                        constexpr int G = decltype(windows)::value;
+                        int u[G];
+                        unsigned cm[G];
+#pragma unroll
+                        for (int j = 0; j < G; ++j) u[j] = M.tour[min(q + 32 * j + lane, n - 1)];
+#pragma unroll
+                        for (int j = 0; j < G; ++j) {
+                            const bool clear = (q + 32 * j + lane < n) & (u[j] != cur) & (M.dlb[u[j]] == 0);
+                            cm[j] = __ballot_sync(FULL2, clear);
+                        }
+#pragma unroll
+                        for (int j = 0; j < G; ++j)
+                            if (cm[j]) {
+                                const int d = cnt + __popc(cm[j] & ((1u << lane) - 1u));
+                                const int slot = ((cm[j] >> lane) & 1u) && d < W ? d : LS_WARPS_MAX;
+                                M.coop[LS_ST + slot] = u[j];
+                                M.coop[LS_POS + slot] = q + 32 * j + lane;
+                                cnt += __popc(cm[j]);
+                            }
+                        q += 32 * G;
+                    };
+                    if (cnt < W && q < n) gather(LsInt<2>{});
+                    while (cnt < W && q < n) gather(LsInt<8>{});
+                    __syncwarp();
+                    cnt = min(cnt, W);
+                    if (lane < cnt) { city = M.coop[LS_ST + lane]; where = M.coop[LS_POS + lane]; }
+                } else {
+                    for (; !cnt && q < n; q += 32) {
+                        const int pp = q + lane;
+                        const int u = pp < n ? M.tour[pp] : 0;
+                        const unsigned cm = __ballot_sync(FULL2, pp < n && !M.dlb[u]);
+                        if (!cm) continue;
+                        where = q + __ffs(cm) - 1;
+                        city = __shfl_sync(FULL2, u, __ffs(cm) - 1);
+                        cnt = 1;
+                    }
+                }
+                if (!cnt) break;
+                LsMove F;
+                int f = 0;            // the first of them with a possible move
+                if (AHEAD && cnt > 1) {
+                    if (lane == 0) { M.coop[0] = 2; M.coop[1] = cnt; }
+                    __syncwarp();
+                    ls_coop_bar(M.coop_warps);
+                    ls_coop_scan(M, n, K, THREE);
+                    ls_coop_bar(M.coop_warps);
+                    const unsigned hm = __ballot_sync(FULL2, lane < cnt && M.coop[LS_MOVES + 8 * (lane < cnt ? lane : 0)] != 0);
+                    f = hm ? __ffs(hm) - 1 : cnt;
+                    const int *o = M.coop + LS_MOVES + 8 * (hm ? f : 0);
+                    F.st = hm ? o[0] : 0;
+                    F.r = o[1];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) F.c[k] = o[2 + k];
+                } else {
+                    F = scan(__shfl_sync(FULL2, city, 0));
+                    f = F.st ? 0 : cnt;
+                }
+                if (lane < cnt && lane < f) M.dlb[city] = 1;      // examined, no move
+                __syncwarp();
+                if (!F.st) {          // none of them moves
+                    p = __shfl_sync(FULL2, where, cnt - 1) + 1;
+                    cur = -1;
+                    continue;
+                }
+                const int a = __shfl_sync(FULL2, city, f);
+                p = __shfl_sync(FULL2, where, f) + 1;
+                bool moved = true;
+                if (F.st == 1) apply(F);
+                else moved = exact(a);
+                if (moved) {
+                    improved = true;
+                    ++round_moves;
+                    ++moves;
+                    cur = a;
+                } else {
+                    if (lane == 0) M.dlb[a] = 1;
+                    __syncwarp();
+                    cur = -1;
+                }
+            }
+        }
+    } while (round_moves > 0 && moves < max_moves);
 }
 
 // warp 0: releases the helper warps (the final arrival of the protocol)
@@ -267,13 +456,12 @@ __device__ __forceinline__ void ls_coop_end(const LsMem &M)
     ls_coop_bar(M.coop_warps);
 }
 
-// reverse so that (x, succ x), (y, succ y) become (x, y), (succ x, succ y);
-// the inner edges of the reversed range swap, the two new edges get dxy, dss
-__device__ __forceinline__ void apply_succ_move(const LsMem &M, int n, int x, int y, float dxy, float dss)
+// the shorter range whose reversal turns (x, succ x), (y, succ y) into (x, y),
+// (succ x, succ y)
+__device__ __forceinline__ void ls_move_range(const LsMem &M, int n, int x, int y, int &i0, int &len)
 {
-    const int lane = threadIdx.x & 31;
-    int i0 = wrap_next(M.pos[x], n);
-    int len = M.pos[y] - i0;
+    i0 = wrap_next(M.pos[x], n);
+    len = M.pos[y] - i0;
     if (len < 0) len += n;
     len += 1;
     if (2 * len > n) {
@@ -282,16 +470,17 @@ __device__ __forceinline__ void apply_succ_move(const LsMem &M, int n, int x, in
         if (len < 0) len += n;
         len += 1;
     }
+}
+
+// one warp alone: reverses, the inner edges of the range swap, the two new
+// edges get dxy, dss
+__device__ __forceinline__ void apply_succ_move(const LsMem &M, int n, int x, int y, float dxy, float dss)
+{
+    const int lane = threadIdx.x & 31;
+    int i0, len;
+    ls_move_range(M, n, x, y, i0, len);
     __syncwarp();
-    if (M.coop && len >= LS_COOP_LEN) {
-        if (lane == 0) { M.coop[0] = 1; M.coop[1] = i0; M.coop[2] = len; }
-        __syncwarp();
-        ls_coop_bar(M.coop_warps);
-        ls_reverse_part(M, n, i0, len, lane, 32 * M.coop_warps);
-        ls_coop_bar(M.coop_warps);
-    } else {
-        ls_reverse_part(M, n, i0, len, lane, 32);
-    }
+    ls_reverse_part<true>(M, n, i0, len, lane, 32);
     __syncwarp();
     if (lane == 0) {
         M.el[wrap_prev(i0, n)] = dxy;
@@ -299,6 +488,28 @@ __device__ __forceinline__ void apply_succ_move(const LsMem &M, int n, int x, in
         if (e >= n) e -= n;
         M.el[e] = dss;
     }
+    __syncwarp();
+}
+
+// warp 0 of a block with helpers: makes the move F (ls2_scan) and clears its
+// cities' bits; no edge lengths are kept
+__device__ __forceinline__ void ls2_apply(const LsMem &M, int n, const LsMove &F)
+{
+    const int lane = threadIdx.x & 31;
+    int i0, len;
+    if (F.r == 0) ls_move_range(M, n, F.c[0], F.c[2], i0, len);
+    else ls_move_range(M, n, F.c[1], F.c[3], i0, len);
+    __syncwarp();
+    if (len >= LS_COOP_LEN) {
+        if (lane == 0) { M.coop[0] = 1; M.coop[1] = i0; M.coop[2] = len; }
+        __syncwarp();
+        ls_coop_bar(M.coop_warps);
+        ls_reverse_part<false>(M, n, i0, len, lane, 32 * M.coop_warps);
+        ls_coop_bar(M.coop_warps);
+    } else {
+        ls_reverse_part<false>(M, n, i0, len, lane, 32);
+    }
+    if (lane < 4) M.dlb[lane == 0 ? F.c[0] : lane == 1 ? F.c[1] : lane == 2 ? F.c[2] : F.c[3]] = 0;
     __syncwarp();
 }
 
@@ -322,8 +533,8 @@ __device__ __forceinline__ int ls_first_may_move(const DevInst &I, const LsMem &
         an1 = M.tour[pv];
         da0 = M.el[pp];
         da1 = M.el[pv];
-        ls_prefetch_row(I.nbr + (size_t)al * K, K * 4);      // read by the work items below
-        const float *nd = I.nbrd32 + (size_t)al * K;
+        ls_prefetch_row(M.nbr + (size_t)al * K, K * 4);      // read by the work items below
+        const float *nd = M.nbrd32 + (size_t)al * K;
         for (int k0 = 0; k0 < K; k0 += 4) {
             float lim[4];
 #pragma unroll
@@ -346,20 +557,6 @@ __device__ __forceinline__ int ls_first_may_move(const DevInst &I, const LsMem &
     }
     const int excl = incl - cnt;
     const int total = __shfl_sync(FULL2, incl, 31);
-    if (M.coop && total > 32) {    // more than one round: shared with the helper warps
-        int *st = M.coop + LS_ST;
-        st[lane] = al;
-        st[32 + lane] = an0;
-        st[64 + lane] = an1;
-        st[96 + lane] = c0;
-        st[128 + lane] = incl;
-        st[160 + lane] = __float_as_int(da0);
-        st[192 + lane] = __float_as_int(da1);
-        if (lane == 0) { M.coop[0] = 2; M.coop[1] = total; }
-        __syncwarp();
-        ls_coop_bar(M.coop_warps);
-        return ls_pretest_rounds(I, M, n, K, total);
-    }
     for (int base = 0; base < total; base += 32) {
         const int t = base + lane;
         int c = 0;      // the lane whose city owns item t: the number of lanes with incl <= t
@@ -433,27 +630,6 @@ __device__ __forceinline__ bool ls_find_move(const DevInst &I, const LsMem &M, i
     return true;
 }
 
-// Command 3, warp 1: the predecessor direction of city a, written to coop.
-__device__ __forceinline__ void ls_pred_search(const DevInst &I, const LsMem &M, int a)
-{
-    const int lane = threadIdx.x & 31, K = I.ls_k;
-    const int nb = lane < K ? I.nbr[(size_t)a * K + lane] : 0;
-    const float nd32 = lane < K ? I.nbrd32[(size_t)a * K + lane] : 0.0f;
-    const double nd64 = lane < K ? I.nbrd[(size_t)a * K + lane] : 0.0;
-    int an = 0, b = 0, bn = 0;
-    float dab = 0.0f, dn = 0.0f;
-    const bool found = ls_find_move(I, M, I.n, K, a, 1, nb, nd32, nd64, an, b, bn, dab, dn);
-    if (lane == 0) {
-        M.coop[3] = found ? 1 : 0;
-        M.coop[4] = an;
-        M.coop[5] = b;
-        M.coop[6] = bn;
-        M.coop[7] = __float_as_int(dab);
-        M.coop[8] = __float_as_int(dn);
-    }
-    __syncwarp();
-}
-
 // Improves `tour` (global memory) in place.  M holds the working arrays; when
 // M.tour is not `tour`, the tour is copied in and back out.  The array
 // pointers are copied into a local first: the search stores through generic
@@ -494,8 +670,8 @@ static __device__ __noinline__ void warp_two_opt(const DevInst &I, int32_t *tour
                     // lists of the 32 positions after them are warmed for the next test
                     if (pp + 32 < n) {
                         const int ah = M.tour[pp + 32];
-                        ls_prefetch_row(I.nbrd32 + (size_t)ah * K, K * 4);
-                        ls_prefetch_row(I.nbr + (size_t)ah * K, K * 4);
+                        ls_prefetch_row(M.nbrd32 + (size_t)ah * K, K * 4);
+                        ls_prefetch_row(M.nbr + (size_t)ah * K, K * 4);
                     }
                     const int f = ls_first_may_move(I, M, n, K, clear, al, pp);
                     if (clear && lane < f) M.dlb[al] = 1;   // examined, no move
@@ -504,33 +680,15 @@ static __device__ __noinline__ void warp_two_opt(const DevInst &I, int32_t *tour
                     p += f;
                 }
                 const int a = M.tour[p];
-                const int nb = lane < K ? I.nbr[(size_t)a * K + lane] : 0;
-                const float nd32 = lane < K ? I.nbrd32[(size_t)a * K + lane] : 0.0f;
+                const int nb = lane < K ? M.nbr[(size_t)a * K + lane] : 0;
+                const float nd32 = lane < K ? M.nbrd32[(size_t)a * K + lane] : 0.0f;
                 const double nd64 = lane < K ? I.nbrd[(size_t)a * K + lane] : 0.0;
                 for (;;) {
                     bool moved = false;
                     int an = 0, b = 0, bn = 0, dir = -1;
                     float dab = 0.0f, dn = 0.0f;
-                    if (M.coop) {   // both directions at once (command 3), successor first
-                        if (lane == 0) { M.coop[0] = 3; M.coop[1] = a; }
-                        __syncwarp();
-                        ls_coop_bar(M.coop_warps);
-                        const bool f0 = ls_find_move(I, M, n, K, a, 0, nb, nd32, nd64, an, b, bn, dab, dn);
-                        ls_coop_bar(M.coop_warps);
-                        if (f0) {
-                            dir = 0;
-                        } else if (M.coop[3]) {
-                            dir = 1;
-                            an = M.coop[4];
-                            b = M.coop[5];
-                            bn = M.coop[6];
-                            dab = __int_as_float(M.coop[7]);
-                            dn = __int_as_float(M.coop[8]);
-                        }
-                    } else {
-                        for (int d = 0; d < 2 && dir < 0; ++d)
-                            if (ls_find_move(I, M, n, K, a, d, nb, nd32, nd64, an, b, bn, dab, dn)) dir = d;
-                    }
+                    for (int d = 0; d < 2 && dir < 0; ++d)
+                        if (ls_find_move(I, M, n, K, a, d, nb, nd32, nd64, an, b, bn, dab, dn)) dir = d;
                     if (dir >= 0) {
                         if (dir == 0) apply_succ_move(M, n, a, b, dab, dn);
                         else apply_succ_move(M, n, an, bn, dn, dab);
@@ -557,14 +715,15 @@ static __device__ __noinline__ void warp_two_opt(const DevInst &I, int32_t *tour
 // the workspace arrays of an instance (no shared memory)
 __device__ __forceinline__ LsMem ls_global(const DevInst &I, int32_t *tour)
 {
-    return LsMem{tour, I.ls_pos, I.ls_dlb, I.ls_el, reinterpret_cast<const float2 *>(I.xy)};
+    return LsMem{tour, I.ls_pos, I.ls_dlb, I.ls_el, reinterpret_cast<const float2 *>(I.xy), I.nbr, I.nbrd32};
 }
 
 // the workspace arrays of ant a's own search (local_search = 2; ant-major tours)
 __device__ __forceinline__ LsMem ls_ant(const DevInst &I, int a)
 {
     const size_t o = (size_t)a * I.n;
-    return LsMem{I.tours + o, I.lsa_pos + o, I.lsa_dlb + o, I.lsa_el + o, reinterpret_cast<const float2 *>(I.xy)};
+    return LsMem{I.tours + o, I.lsa_pos + o, I.lsa_dlb + o, I.lsa_el + o, reinterpret_cast<const float2 *>(I.xy),
+                 I.nbr, I.nbrd32};
 }
 
 // shared memory: tour, pos, el (4n bytes each), dlb (n bytes), then the
@@ -573,9 +732,23 @@ __host__ __device__ inline size_t ls_smem_core(int n) { return (size_t)n * 13; }
 __host__ __device__ inline size_t ls_xy_offset(int n) { return ((size_t)n * 13 + 15) & ~(size_t)15; }
 __host__ __device__ inline size_t ls_smem_full(int n) { return ls_xy_offset(n) + (size_t)n * 8; }
 
+// every array in `sm` (ls_smem_full bytes), the coordinates not yet filled
+__device__ __forceinline__ LsMem ls_shared_full(const DevInst &I, unsigned char *sm)
+{
+    const int n = I.n;
+    LsMem M;
+    M.tour = reinterpret_cast<int32_t *>(sm);
+    M.pos = reinterpret_cast<int32_t *>(sm + (size_t)n * 4);
+    M.el = reinterpret_cast<float *>(sm + (size_t)n * 8);
+    M.dlb = sm + (size_t)n * 12;
+    M.xy = reinterpret_cast<const float2 *>(sm + ls_xy_offset(n));
+    M.nbr = I.nbr;
+    M.nbrd32 = I.nbrd32;
+    return M;
+}
+
 // arrays in `sm` (smem_bytes) where they fit, else `fallback`; one warp
-// (copy = false: the same pointers without filling the coordinates, for the
-// helper warps of a block)
+// (copy = false: the same pointers without filling the coordinates)
 __device__ __forceinline__ LsMem ls_shared(const DevInst &I, int32_t *tour, unsigned char *sm, size_t smem_bytes,
                                            const LsMem &fallback, bool copy = true)
 {
@@ -587,6 +760,8 @@ __device__ __forceinline__ LsMem ls_shared(const DevInst &I, int32_t *tour, unsi
     M.el = reinterpret_cast<float *>(sm + (size_t)n * 8);
     M.dlb = sm + (size_t)n * 12;
     M.xy = reinterpret_cast<const float2 *>(I.xy);
+    M.nbr = I.nbr;
+    M.nbrd32 = I.nbrd32;
     if (I.kind == 0 && ls_smem_full(n) <= smem_bytes) {
         float2 *sxy = reinterpret_cast<float2 *>(sm + ls_xy_offset(n));
         if (copy) {
