@@ -46,7 +46,7 @@ template <int NA>
 __device__ __forceinline__ void warp_ant_lengths(const DevInst &I, const int (&ants)[NA], double (&out)[NA])
 {
     const int lane = threadIdx.x & 31, n = I.n, kp = I.k_pad;
-    const double *__restrict__ cdist = I.cdist;
+    const double *cdist = I.cdist;
     double P[NA];
 #pragma unroll
     for (int h = 0; h < NA; ++h) P[h] = 0.0;
@@ -63,14 +63,16 @@ __device__ __forceinline__ void warp_ant_lengths(const DevInst &I, const int (&a
                 from[h][k] = I.tours[step_ix(I, ants[h], s - 1)];
                 c[h][k] = I.slots[step_ix(I, ants[h], s)];
             }
+        // the address of each edge's length is selected, not the load: loads behind
+        // a lane-dependent branch waited for one another
         double d[NA][U];
 #pragma unroll
         for (int h = 0; h < NA; ++h)
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const int s = e + 32 * k + 1;
-                d[h][k] = c[h][k] != SLOT_FALLBACK ? cdist[(size_t)from[h][k] * kp + c[h][k]]
-                                                   : I.dstep[step_ix(I, ants[h], s)];
+                const double *src = I.dstep + step_ix(I, ants[h], e + 32 * k + 1);
+                if (c[h][k] != SLOT_FALLBACK) src = cdist + ((size_t)from[h][k] * kp + c[h][k]);
+                d[h][k] = *src;
             }
 #pragma unroll
         for (int k = 0; k < U; ++k)
@@ -81,15 +83,11 @@ __device__ __forceinline__ void warp_ant_lengths(const DevInst &I, const int (&a
 #pragma unroll
         for (int h = 0; h < NA; ++h) {
             const int a = ants[h];
-            double d;
-            if (e == n - 1) {
-                d = I.dstep[step_ix(I, a, 0)];            // closing edge
-            } else {
-                const uint8_t c = I.slots[step_ix(I, a, e + 1)];
-                d = c != SLOT_FALLBACK ? cdist[(size_t)I.tours[step_ix(I, a, e)] * kp + c]
-                                       : I.dstep[step_ix(I, a, e + 1)];
-            }
-            P[h] = __dadd_rn(P[h], d);
+            const int s = e == n - 1 ? 0 : e + 1;          // step 0 holds the closing edge
+            const uint8_t c = s ? I.slots[step_ix(I, a, s)] : SLOT_FALLBACK;
+            const double *src = I.dstep + step_ix(I, a, s);
+            if (c != SLOT_FALLBACK) src = cdist + ((size_t)I.tours[step_ix(I, a, e)] * kp + c);
+            P[h] = __dadd_rn(P[h], *src);
         }
     }
 #pragma unroll
