@@ -290,7 +290,7 @@ inline int plan_batch(const hac_instance *ins, const hac_params *ps, int count, 
 
 
 struct FusedGroup {
-    int clog = 0, apw = 4, count = 0, order_off = 0;
+    int clog = 0, apw = 4, ls = 0, count = 0, order_off = 0;
     int rows_cap = 0, kp_cap = 0, stride = 0, warps = 0, block_warps = 0, xy_cap = 0, list_rows = 0;
 };
 
@@ -364,7 +364,7 @@ inline int upload_inputs(const DevInst &D, const hac_instance &in, const Sizes &
     return HAC_OK;
 }
 
-// Groups the given instances by layout: ants per warp and cluster size (the
+// Groups the given instances by layout: local search or none, ants per warp and cluster size (the
 // fewest CTAs whose shared memory holds the instance's share of the
 // candidate table and visited masks, at least 2^clog_min), each group ordered
 // by decreasing work.  apw = 0 stands for 8 ants per warp, on one CTA where the
@@ -412,17 +412,21 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
         if (clog[q] < 0) return HAC_EUNSUPPORTED;
     }
     const int apws[5] = {2, 4, 8, 16, 32};
+    auto in_group = [&](int q, int cl, int a, int ls) {
+        return clog[q] == cl && qapw[q] == a && (zs[members[q]].ls != 0) == (ls != 0);
+    };
     for (;;) {   // group caps may exceed the limit when members differ: move a group up
         groups.clear();
         bool again = false;
         for (int cl = 0; cl <= 3 && !again; ++cl)
-            for (int ai = 0; ai < 5 && !again; ++ai) {
-                const int a = apws[ai];
+            for (int ai = 0; ai < 10 && !again; ++ai) {
+                const int a = apws[ai >> 1], ls = ai & 1;
                 FusedGroup G;
                 G.clog = cl;
                 G.apw = a;
+                G.ls = ls;
                 for (int q = 0; q < count; ++q) {
-                    if (clog[q] != cl || qapw[q] != a) continue;
+                    if (!in_group(q, cl, a, ls)) continue;
                     int rows, warps;
                     fits(q, cl, a, rows, warps);
                     const Sizes &z = zs[members[q]];
@@ -440,14 +444,14 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
                 const size_t base = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, 0, 0);
                 if (base > FUSED_SMEM_LIMIT) {
                     if (cl == 3) return HAC_EUNSUPPORTED;
-                    for (int q = 0; q < count; ++q) if (clog[q] == cl && qapw[q] == a) clog[q] = cl + 1;
+                    for (int q = 0; q < count; ++q) if (in_group(q, cl, a, ls)) clog[q] = cl + 1;
                     again = true;
                     break;
                 }
                 // coordinates of the fallback scan in shared memory when they still fit
                 int nmax = 0;
                 for (int q = 0; q < count; ++q)
-                    if (clog[q] == cl && qapw[q] == a) nmax = std::max(nmax, zs[members[q]].n);
+                    if (in_group(q, cl, a, ls)) nmax = std::max(nmax, zs[members[q]].n);
                 if (base + (size_t)nmax * 8 <= FUSED_SMEM_LIMIT) G.xy_cap = nmax;
                 // and the lookup lists of this CTA's rows
                 if (fallback_list &&
@@ -464,7 +468,7 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
     std::vector<long long> gmax(groups.size(), 0);
     for (size_t g = 0; g < groups.size(); ++g)
         for (int q = 0; q < count; ++q)
-            if (clog[q] == groups[g].clog && qapw[q] == groups[g].apw) gmax[g] = std::max(gmax[g], work(members[q]));
+            if (in_group(q, groups[g].clog, groups[g].apw, groups[g].ls)) gmax[g] = std::max(gmax[g], work(members[q]));
     std::vector<size_t> gi(groups.size());
     for (size_t g = 0; g < gi.size(); ++g) gi[g] = g;
     std::stable_sort(gi.begin(), gi.end(), [&](size_t x, size_t y) { return gmax[x] > gmax[y]; });
@@ -475,7 +479,7 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
     for (FusedGroup &G : groups) {
         G.order_off = (int)order.size();
         std::vector<int32_t> mem;
-        for (int q = 0; q < count; ++q) if (clog[q] == G.clog && qapw[q] == G.apw) mem.push_back(members[q]);
+        for (int q = 0; q < count; ++q) if (in_group(q, G.clog, G.apw, G.ls)) mem.push_back(members[q]);
         std::stable_sort(mem.begin(), mem.end(), [&](int x, int y) { return work(x) > work(y); });
         order.insert(order.end(), mem.begin(), mem.end());
     }
@@ -500,7 +504,7 @@ inline cudaError_t launch_groups(const DevInst *d_inst, const int32_t *d_order, 
     for (size_t g = 0; g < groups.size(); ++g) {
         const FusedGroup &G = groups[g];
         cudaError_t e = launch_fused(d_inst, d_order + G.order_off, d_iters ? d_iters + G.order_off : nullptr,
-                                     G.count, G.clog, G.apw, G.warps, G.block_warps,
+                                     G.count, G.clog, G.apw, G.ls != 0, G.warps, G.block_warps,
                                      G.rows_cap, G.kp_cap, G.stride, G.xy_cap, G.list_rows, iters, s, g > 0);
         if (e != cudaSuccess && err == cudaSuccess) err = e;
     }

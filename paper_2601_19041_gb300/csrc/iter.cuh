@@ -5,7 +5,7 @@
 //                    L_gb and bounds (eq. tau_init / tau_min_nols from L_gb);
 //                    the elite T+ (T_ib, or T_rb every u_gb iterations) and
 //                    its succ/pred; trace; t+1
-//   update_slot      tau <- min(tau_max, max(tau_min, fl32(tau*(1-rho))
+//   update_slots4    tau <- min(tau_max, max(tau_min, fl32(tau*(1-rho))
 //                    [+ fl32(1/L(T+)) on T+ edges])) (eqs. pheromone_update,
 //                    pheromone_delta) and choice = fl32(tau^alpha * W)
 //   schedule end     (schedule = 1) every 100 iterations, when T_rb has not
@@ -218,16 +218,28 @@ __device__ __forceinline__ void block_schedule_end(const DevInst &I, InstState *
     __syncthreads();
 }
 
-// new tau of real slot s = (i, c) with candidate j; writes tau, returns choice
-__device__ __forceinline__ float update_slot(const DevInst &I, size_t s, int i, int j, float omega,
-                                             float delta, float tmin, float tmax)
+// new tau and choice of the four slots s .. s+3 of row i (one 16-byte access per
+// array; rows are multiples of 4 slots) with candidates j; padding slots (j
+// not a node) keep what they hold
+__device__ __forceinline__ float4 update_slots4(const DevInst &I, size_t s, int i, const int (&j)[4], float4 old_choice,
+                                                float omega, float delta, float tmin, float tmax)
 {
-    float x = __fmul_rn(I.tau[s], omega);
-    if (I.succ[i] == j || (I.kind == 0 && I.pred[i] == j)) x = __fadd_rn(x, delta);
-    const float y = x > tmin ? x : tmin;
-    const float tau = y < tmax ? y : tmax;
-    I.tau[s] = tau;
-    return choice_value(I, tau, I.W[s]);
+    const float4 t4 = *reinterpret_cast<const float4 *>(I.tau + s), w4 = *reinterpret_cast<const float4 *>(I.W + s);
+    const int sc = I.succ[i], pr = I.kind == 0 ? I.pred[i] : -1;
+    float t[4] = {t4.x, t4.y, t4.z, t4.w}, c[4] = {old_choice.x, old_choice.y, old_choice.z, old_choice.w};
+    const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float x = __fmul_rn(t[q], omega);
+        x = sc == j[q] || pr == j[q] ? __fadd_rn(x, delta) : x;
+        const float y = x > tmin ? x : tmin;
+        const float tau = y < tmax ? y : tmax;
+        const bool real = j[q] >= 0 && j[q] < I.n;
+        t[q] = real ? tau : t[q];
+        c[q] = real ? choice_value(I, tau, w[q]) : c[q];
+    }
+    *reinterpret_cast<float4 *>(I.tau + s) = make_float4(t[0], t[1], t[2], t[3]);
+    return make_float4(c[0], c[1], c[2], c[3]);
 }
 
 }  // namespace hac

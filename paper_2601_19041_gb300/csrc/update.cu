@@ -25,19 +25,21 @@ __global__ void k_gb(const DevInst *insts)
     block_global_best(I, st);
 }
 
+// four slots a thread: 1024 slots of an instance per block of 256 threads
 __global__ void k_update(const DevInst *insts, const int2 *slotmap)
 {
     const int2 sm = slotmap[blockIdx.x];
     const DevInst &I = insts[sm.x];
     const InstState *st = I.st;
     if (!st->active) return;
-    const size_t s = (size_t)sm.y + threadIdx.x;
+    const size_t s = (size_t)sm.y + 4 * threadIdx.x;
     if (s >= (size_t)I.n * I.k_pad) return;
-    const int j = I.cand[s];
-    if (j < 0) return;
+    const int4 j4 = *reinterpret_cast<const int4 *>(I.cand + s);
+    const int j[4] = {j4.x, j4.y, j4.z, j4.w};
     const float omega = __double2float_rn(__dsub_rn(1.0, I.rho));
     const float delta = __double2float_rn(__ddiv_rn(1.0, st->L_dep));
-    I.choice[s] = update_slot(I, s, (int)(s / I.k_pad), j, omega, delta, st->tau_min, st->tau_max);
+    float4 *ch = reinterpret_cast<float4 *>(I.choice + s);
+    *ch = update_slots4(I, s, (int)(s / I.k_pad), j, *ch, omega, delta, st->tau_min, st->tau_max);
 }
 
 // MMAS schedule end (restart check, next u_gb); one block per instance
@@ -59,7 +61,7 @@ int launch_iteration_tail(const DevInst *d_inst, int count, const int2 *d_slotma
     k_select<<<count, 256, 0, s>>>(d_inst);
     if (any_ls) launch_two_opt_ib(d_inst, count, max_n, s);
     k_gb<<<count, 256, 0, s>>>(d_inst);
-    k_update<<<slotmap_len, 1024, 0, s>>>(d_inst, d_slotmap);
+    k_update<<<slotmap_len, 256, 0, s>>>(d_inst, d_slotmap);
     k_schedule<<<count, 256, 0, s>>>(d_inst);
     return (any_ls ? 5 : 4) + (ls_all_m > 0 ? 1 : 0);
 }
