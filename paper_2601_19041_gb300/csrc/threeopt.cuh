@@ -607,9 +607,8 @@ static __device__ __forceinline__ void warp_two_opt_any(const DevInst &I, int32_
 
 // Improves `tour` (global memory) in place; M as for warp_two_opt (its el
 // array serves as the scratch of the middle rewrite).
-static __device__ __noinline__ void warp_three_opt(const DevInst &I, int32_t *tour, const LsMem &Mref)
+__device__ __forceinline__ void warp_three_opt_body(const DevInst &I, int32_t *tour, const LsMem &M)
 {
-    const LsMem M = Mref;   // a local copy: see warp_two_opt
     const int lane = threadIdx.x & 31;
     const int n = I.n, K = I.ls_k;
     if (M.tour != tour)
@@ -622,6 +621,13 @@ static __device__ __noinline__ void warp_three_opt(const DevInst &I, int32_t *to
     if (M.tour != tour)
         for (int p = lane; p < n; p += 32) tour[p] = M.tour[p];
     __syncwarp();
+}
+
+// the same as a call (the cluster kernel)
+static __device__ __noinline__ void warp_three_opt(const DevInst &I, int32_t *tour, const LsMem &Mref)
+{
+    const LsMem M = Mref;
+    warp_three_opt_body(I, tour, M);
 }
 
 // The search of a symmetric instance by a whole block (every thread calls it):

@@ -20,9 +20,9 @@
 // Moves follow the FP64 gain (d_ij as in the length, gain = (d(a,dir a) -
 // d(a,b)) + d(b,dir b) - d(dir a,dir b)), but most candidates are decided from
 // FP32 copies: el[p] holds d(tour[p], tour[p+1]) in FP32 and nbrd32 the
-// neighbour distances.  Each FP32 distance is within 4 units of 2^-24 (relative) of the
+// neighbour distances.  Each FP32 distance is within 5 units of 2^-24 (relative) of the
 // FP64 one, so the FP32 estimate of the four-term gain is within about
-// 8 * 2^-24 of the sum of the four magnitudes.  With tol = 4e-6 times that
+// 9 * 2^-24 of the sum of the four magnitudes.  With tol = 4e-6 times that
 // sum (plus 1e-18 for FP32 underflow), an estimate below 1e-10 - tol means the
 // FP64 gain is certainly <= 1e-10, one above 1e-10 + tol that it is certainly
 // above; only estimates in between are decided in FP64.  Likewise d(a, b) is
@@ -116,6 +116,16 @@ __device__ __forceinline__ float ls_d32(const float2 *xy, int u, int v)
     return __fsqrt_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)));
 }
 
+// FP32 distance with the approximate square root (error at most 2^-23 of it):
+// within 5 units of 2^-24, far inside the 4e-6 bands
+__device__ __forceinline__ float ls_da32(float2 p, float2 q)
+{
+    const float dx = __fsub_rn(q.x, p.x), dy = __fsub_rn(q.y, p.y);
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy))));
+    return r;
+}
+
 // the FP64 gain from FP32 estimates of its terms: 0 certainly <= LS_GAIN,
 // 2 certainly above, 1 undecided
 __device__ __forceinline__ int ls_gain_class(float da, float dab, float dbb, float dn)
@@ -193,7 +203,7 @@ __device__ __forceinline__ bool ls_item_may_improve(const DevInst &I, const LsMe
     const int pb = M.pos[b];
     const int pe = dir == 0 ? pb : wrap_prev(pb, n);     // the edge (b, dir b)
     const int bn = M.tour[dir == 0 ? wrap_next(pb, n) : pe];
-    return b != an && bn != a && ls_may_improve(da, dab, M.el[pe], ls_d32(M.xy, an, bn));
+    return b != an && bn != a && ls_may_improve(da, dab, M.el[pe], ls_da32(M.xy[an], M.xy[bn]));
 }
 
 // What the examination of a city in FP32 found: st 0 no move; 1 the city's
@@ -206,16 +216,6 @@ struct LsMove {
 
 __device__ __forceinline__ LsMove ls3_scan(const LsMem &M, int n, int K, int a);
 __device__ __forceinline__ void ls3_coop_rewrite(const LsMem &M);
-
-// FP32 distance with the approximate square root (error at most 2^-23 of it):
-// within 5 units of 2^-24, far inside the 4e-6 bands
-__device__ __forceinline__ float ls_da32(float2 p, float2 q)
-{
-    const float dx = __fsub_rn(q.x, p.x), dy = __fsub_rn(q.y, p.y);
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy))));
-    return r;
-}
 
 // One city's 2-opt moves in FP32 (whole warp, only reads, the same result in
 // every lane): a neighbour per lane, both directions.
@@ -599,7 +599,7 @@ __device__ __forceinline__ bool ls_find_move(const DevInst &I, const LsMem &M, i
         bbn = dir == 0 ? M.tour[wrap_next(pb, n)] : M.tour[wrap_prev(pb, n)];
         if (!(bb == an || bbn == a)) {
             const float dbb = M.el[dir == 0 ? pb : wrap_prev(pb, n)];
-            dnn = ls_d32(M.xy, an, bbn);
+            dnn = ls_da32(M.xy[an], M.xy[bbn]);
             const int g = ls_gain_class(da32, nd32, dbb, dnn);
             cand = g != 0;
             sure = g == 2 && __fmul_rn(da32, LS_G1_LO) > nd32;   // and d(a, b) < d(a, dir a) for certain
@@ -635,9 +635,8 @@ __device__ __forceinline__ bool ls_find_move(const DevInst &I, const LsMem &M, i
 // pointers are copied into a local first: the search stores through generic
 // pointers, and pointers read through a reference would be reloaded after
 // every store.
-static __device__ __noinline__ void warp_two_opt(const DevInst &I, int32_t *tour, const LsMem &Mref)
+__device__ __forceinline__ void warp_two_opt_body(const DevInst &I, int32_t *tour, const LsMem &M)
 {
-    const LsMem M = Mref;
     const int lane = threadIdx.x & 31;
     const int n = I.n, K = I.ls_k;
     if (M.tour != tour)
@@ -710,6 +709,13 @@ static __device__ __noinline__ void warp_two_opt(const DevInst &I, int32_t *tour
     if (M.tour != tour)
         for (int p = lane; p < n; p += 32) tour[p] = M.tour[p];
     __syncwarp();
+}
+
+// the same as a call (the cluster kernel)
+static __device__ __noinline__ void warp_two_opt(const DevInst &I, int32_t *tour, const LsMem &Mref)
+{
+    const LsMem M = Mref;
+    warp_two_opt_body(I, tour, M);
 }
 
 // the workspace arrays of an instance (no shared memory)
