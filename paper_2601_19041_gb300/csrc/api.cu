@@ -26,8 +26,8 @@ struct BatchPart {
     int b0 = 0, count = 0;                 // instances b0 .. b0+count-1
     int warp_off = 0, warp_len = 0;        // slice of the warp table (instance index relative to b0)
     int slot_off = 0, slot_len = 0;        // slice of the relative slot table
-    int max_n = 0, max_kp = 0, max_m = 0, ls_all_m = 0;
-    bool any_ls = false;
+    int max_n = 0, max_kp = 0, max_m = 0;
+    TailNeeds needs;
     cudaStream_t stream = nullptr;         // the batch's stream when there is one part
     cudaEvent_t fork = nullptr, join = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -53,8 +53,6 @@ struct hac_batch {
     std::vector<FusedGroup> groups;   // non-empty when the fused kernel is used
     int *d_err = nullptr;
     int max_n = 0, max_kp = 0;
-    bool any_ls = false;
-    int ls_all_m = 0;               // largest m among the instances with local search on every ant
     std::vector<int> t_host;
     cudaGraphExec_t fexec = nullptr;   // fused groups (fork/join included) for fexec_iters iterations
     int fexec_iters = -1;
@@ -163,8 +161,6 @@ static int batch_setup(hac_batch *bt, const hac_instance *ins, const hac_params 
         }
         bt->max_n = std::max(bt->max_n, z.n);
         bt->max_kp = std::max(bt->max_kp, z.kp);
-        bt->any_ls |= z.ls != 0;
-        if (z.ls == 2 || z.ls == 4) bt->ls_all_m = std::max(bt->ls_all_m, z.m);
     }
     // parts of the per-step path: contiguous instance ranges of about equal work
     const int nparts = std::max(1, std::min(std::min((int)bt->ex.parts, 64), count));
@@ -209,8 +205,7 @@ static int batch_setup(hac_batch *bt, const hac_instance *ins, const hac_params 
             pt.max_n = std::max(pt.max_n, z.n);
             pt.max_kp = std::max(pt.max_kp, z.kp);
             pt.max_m = std::max(pt.max_m, z.m);
-            pt.any_ls |= z.ls != 0;
-            if (z.ls == 2 || z.ls == 4) pt.ls_all_m = std::max(pt.ls_all_m, z.m);
+            add_needs(pt.needs, z);
         }
         pt.warp_len = (int)warpmap.size() - pt.warp_off;
         pt.slot_len = (int)slotrel.size() - pt.slot_off;
@@ -358,15 +353,15 @@ static int enqueue_iteration(hac_batch *bt, const BatchPart &pt)
     if (bt->parts.size() > 1)   // several parts: no per-group timing (the fork/join region is timed)
         return launch_construct(d, bt->d_warpmap + pt.warp_off, pt.warp_len, bt->ex.ants_per_warp,
                                 bt->ex.warps_per_block, pt.max_n, pt.max_kp, pt.max_m, pt.count, pt.stream) +
-               launch_iteration_tail(d, pt.count, bt->d_slotmap_rel + pt.slot_off, pt.slot_len, pt.any_ls,
-                                     pt.max_n, pt.ls_all_m, pt.stream);
+               launch_iteration_tail(d, pt.count, bt->d_slotmap_rel + pt.slot_off, pt.slot_len, pt.needs,
+                                     pt.max_n, pt.stream);
     int k = timed(bt, 0, [&] {
         return launch_construct(d, bt->d_warpmap + pt.warp_off, pt.warp_len, bt->ex.ants_per_warp,
                                 bt->ex.warps_per_block, pt.max_n, pt.max_kp, pt.max_m, pt.count, pt.stream);
     });
     k += timed(bt, 1, [&] {
-        return launch_iteration_tail(d, pt.count, bt->d_slotmap_rel + pt.slot_off, pt.slot_len, pt.any_ls,
-                                     pt.max_n, pt.ls_all_m, pt.stream);
+        return launch_iteration_tail(d, pt.count, bt->d_slotmap_rel + pt.slot_off, pt.slot_len, pt.needs,
+                                     pt.max_n, pt.stream);
     });
     return k;
 }

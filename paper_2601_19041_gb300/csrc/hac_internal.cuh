@@ -257,8 +257,14 @@ int launch_prep(const DevInst *d_inst, const DevInst *h_inst, int count, const i
                 cudaStream_t s);
 int launch_construct(const DevInst *d_inst, const int4 *d_warpmap, int warpmap_len, int apw,
                      int warps_per_block, int max_n, int max_kp, int max_m, int count, cudaStream_t s);
-int launch_iteration_tail(const DevInst *d_inst, int count, const int2 *d_slotmap,
-                          int slotmap_len, bool any_ls, int max_n, int ls_all_m, cudaStream_t s);
+// what the end of an iteration has to do for some instance of a launch
+struct TailNeeds {
+    bool ls_ib = false;      // local search on the iteration-best tour
+    bool schedule = false;   // the MMAS schedule
+    int ls_all_m = 0;        // largest m with local search on every ant (0: none)
+};
+int launch_iteration_tail(const DevInst *d_inst, int count, const int2 *d_slotmap, int slotmap_len,
+                          const TailNeeds &needs, int max_n, cudaStream_t s);
 // fused cluster kernel (fused.cuh, fused.cu): one cluster of 2^clog CTAs per instance;
 // d_iters (parallel to d_order, may be null) gives each cluster its own
 // iteration count instead of `iters`

@@ -56,7 +56,7 @@ struct Arena {
 };
 
 struct Sizes {
-    int n, kind, kp, k_eff, m, iters, ls, ls_k, sym, half;
+    int n, kind, kp, k_eff, m, iters, ls, ls_k, sym, half, schedule;
     long long nnz;
 };
 
@@ -169,12 +169,21 @@ inline int instance_sizes(const hac_instance &in, const hac_params &p, int on_de
     z.ls_k = p.local_search ? p.ls_k : 0;
     z.sym = in.symmetrize;
     z.half = in.h_dtype;
+    z.schedule = p.schedule;
     const long long last = in.h_nnz;
     if (last < 0 || last > (1LL << 31) - 1) return HAC_EINVAL;
     if (!on_dev && in.h_rowptr[in.n] != last) return HAC_EINVAL;
     if (last > 0 && (!in.h_col || !in.h_val)) return HAC_EINVAL;
     z.nnz = last;
     return HAC_OK;
+}
+
+// adds what instance z needs at the end of an iteration
+inline void add_needs(TailNeeds &t, const Sizes &z)
+{
+    t.ls_ib |= z.ls == 1 || z.ls == 3;
+    t.schedule |= z.schedule != 0;
+    if (z.ls == 2 || z.ls == 4) t.ls_all_m = std::max(t.ls_all_m, z.m);
 }
 
 // Replays the same sequence of slices for sizing and for binding pointers.

@@ -300,8 +300,7 @@ int enqueue_step_route(hac_server *sv, const std::vector<int> &mem, int par)
     int2 *hs = sv->h_sslot[par];
     size_t nw = 0, ns = 0;
     int it = sv->cfg.iters_per_tick, max_n = 0, max_kp = 0, max_m = 0;
-    bool any_ls = false;
-    int ls_all_m = 0;
+    TailNeeds needs;
     for (size_t b = 0; b < mem.size(); ++b) {
         const Slot &S = sv->slots[mem[b]];
         hI[b] = sv->hi[mem[b]];
@@ -312,8 +311,7 @@ int enqueue_step_route(hac_server *sv, const std::vector<int> &mem, int par)
         max_n = std::max(max_n, S.z.n);
         max_kp = std::max(max_kp, S.z.kp);
         max_m = std::max(max_m, S.z.m);
-        any_ls |= S.z.ls != 0;
-        if (S.z.ls == 2 || S.z.ls == 4) ls_all_m = std::max(ls_all_m, S.z.m);
+        add_needs(needs, S.z);
     }
     const int count = (int)mem.size();
     cudaStream_t ss = sv->sstream;
@@ -325,8 +323,7 @@ int enqueue_step_route(hac_server *sv, const std::vector<int> &mem, int par)
     for (int q = 0; q < it; ++q) {
         sv->launches += launch_construct(sv->d_sinst[par], sv->d_swarp[par], (int)nw, apw,
                                          sv->sex.warps_per_block, max_n, max_kp, max_m, count, ss);
-        sv->launches += launch_iteration_tail(sv->d_sinst[par], count, sv->d_sslot[par], (int)ns, any_ls, max_n,
-                                              ls_all_m, ss);
+        sv->launches += launch_iteration_tail(sv->d_sinst[par], count, sv->d_sslot[par], (int)ns, needs, max_n, ss);
     }
     CK(cudaGetLastError());
     for (int q : mem) sv->slots[q].t += it;
