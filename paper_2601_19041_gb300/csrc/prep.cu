@@ -246,7 +246,14 @@ __device__ __forceinline__ void warp_min_kj(float &k, int &j)
 // that provably contains the exact K smallest; each of those distances is
 // computed once (up to CACHE per lane, recomputed beyond).  Cost instances
 // order by the FP32 cost directly (its FP64 widening is exact and monotone).
-constexpr int CACHE = 4;
+//
+// One pass over the nodes: every lane keeps its KEEP smallest keys, and the K
+// smallest of all are then taken head by head (two warp reductions each).  When
+// a lane has used up all it kept (for K = 20, one row in a thousand) its next
+// node is unknown and the row is done again with a pass over the nodes per
+// neighbour, as all rows were before (n = 10000, 20 neighbours of 80000 nodes:
+// 18.0 ms, about 4 ms now).
+constexpr int CACHE = 4, KEEP = 6;
 
 template <typename Pred>
 __device__ void warp_knn(const DevInst &I, int i, int K, Pred pred, double &dout, int &jout)
@@ -257,20 +264,64 @@ __device__ void warp_knn(const DevInst &I, int i, int K, Pred pred, double &dout
     auto key = [&](int u) -> float {
         return I.kind == 0 ? key32_xy(pi, xy[u]) : I.cost[(size_t)i * I.n + u];
     };
-    // pass 1: K-th smallest (key, u)
+    float rk[KEEP];
+    int ru[KEEP], seen_all = 0;
+#pragma unroll
+    for (int c = 0; c < KEEP; ++c) { rk[c] = __int_as_float(0x7f800000); ru[c] = 0x7fffffff; }
+#pragma unroll 4
+    for (int u = lane; u < I.n; u += 32) {
+        if (u == i || !pred(u)) continue;
+        const float kk = key(u);
+        ++seen_all;
+        if (kk < rk[KEEP - 1]) {               // ascending u: an equal key stays behind
+            rk[KEEP - 1] = kk;
+            ru[KEEP - 1] = u;
+#pragma unroll
+            for (int c = KEEP - 1; c > 0; --c)
+                if (rk[c] < rk[c - 1]) {
+                    const float tk = rk[c]; rk[c] = rk[c - 1]; rk[c - 1] = tk;
+                    const int tu = ru[c]; ru[c] = ru[c - 1]; ru[c - 1] = tu;
+                }
+        }
+    }
+    // K-th smallest (key, u)
     float pk = -1.0f;
     int pu = -1;
-    for (int r = 0; r < K; ++r) {
-        float bk = __int_as_float(0x7f800000);
-        int bu = 0x7fffffff;
-        for (int u = lane; u < I.n; u += 32) {
-            if (u == i || !pred(u)) continue;
-            float kk = key(u);
-            if (key_less(pk, pu, kk, u) && key_less(kk, u, bk, bu)) { bk = kk; bu = u; }
+    int used = 0;
+    bool known = true;                         // this lane's head is its smallest unused node
+    for (int r = 0; r < K && known; ++r) {
+        float hk = __int_as_float(0x7f800000);
+        int hu = 0x7fffffff;
+#pragma unroll
+        for (int c = 0; c < KEEP; ++c) if (c == used) { hk = rk[c]; hu = ru[c]; }
+        const unsigned ok = hu == 0x7fffffff ? 0xffffffffu : ord_key(hk);
+        const unsigned wk = __reduce_min_sync(FULL, ok);
+        const int wu = (int)__reduce_min_sync(FULL, ok == wk ? (unsigned)hu : 0x7fffffffu);
+        const unsigned owner = __ballot_sync(FULL, hu == wu && hu != 0x7fffffff);
+        if (!owner) { pk = __int_as_float(0x7f800000); pu = 0x7fffffff; known = false; break; }
+        const float wf = __shfl_sync(FULL, hk, __ffs(owner) - 1);
+        if (hu == wu) ++used;
+        if (I.kind == 1 && lane == r) { dout = (double)wf; jout = wu; }
+        pk = wf;
+        pu = wu;
+        if (r + 1 < K) known = !__any_sync(FULL, used == KEEP && seen_all > KEEP);
+    }
+    if (!known) {
+        pk = -1.0f;
+        if (I.kind == 1) pk = __int_as_float(0xff800000);   // costs may be negative
+        pu = -1;
+        for (int r = 0; r < K; ++r) {
+            float bk = __int_as_float(0x7f800000);
+            int bu = 0x7fffffff;
+            for (int u = lane; u < I.n; u += 32) {
+                if (u == i || !pred(u)) continue;
+                float kk = key(u);
+                if (key_less(pk, pu, kk, u) && key_less(kk, u, bk, bu)) { bk = kk; bu = u; }
+            }
+            warp_min_kj(bk, bu);
+            if (I.kind == 1 && lane == r) { dout = (double)bk; jout = bu; }
+            pk = bk; pu = bu;
         }
-        warp_min_kj(bk, bu);
-        if (I.kind == 1 && lane == r) { dout = (double)bk; jout = bu; }
-        pk = bk; pu = bu;
     }
     if (I.kind == 1) return;
     float thr = __fadd_rn(__fmul_rn(pk, 1.00001f), 1e-30f);
@@ -279,7 +330,20 @@ __device__ void warp_knn(const DevInst &I, int i, int K, Pred pred, double &dout
     int cu[CACHE];
     int nc = 0;
     bool ovf = false;
-    for (int u = lane; u < I.n; u += 32) {
+    // from the kept keys when every lane kept all of its nodes inside the margin
+    int within = 0;
+#pragma unroll
+    for (int c = 0; c < KEEP; ++c) within += ru[c] != 0x7fffffff && rk[c] <= thr;
+    const bool kept = known && __all_sync(FULL, within <= CACHE && (seen_all <= KEEP || rk[KEEP - 1] > thr));
+    if (kept) {
+#pragma unroll
+        for (int c = 0; c < CACHE; ++c) {
+            if (c < within) { cd[c] = dist64(I, i, ru[c]); cu[c] = ru[c]; }
+            else { cd[c] = DINF; cu[c] = 0x7fffffff; }
+        }
+        nc = within;
+    }
+    for (int u = kept ? I.n : lane; u < I.n; u += 32) {
         if (u == i || !pred(u) || !(key(u) <= thr)) continue;
         if (nc < CACHE) {
 #pragma unroll
