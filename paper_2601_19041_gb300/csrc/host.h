@@ -416,8 +416,10 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
                 continue;
             }
         }
-        for (int cl = clog_min; cl <= 3; ++cl)
-            if (fits(q, cl, qapw[q], rows, warps)) { clog[q] = cl; break; }
+        // (apw = 0: where masks for whole warps of 8 ants do not fit, 4 or 2)
+        for (int a = qapw[q]; a && clog[q] < 0; a = apw == 0 && a > 2 ? a / 2 : 0)
+            for (int cl = clog_min; cl <= 3; ++cl)
+                if (fits(q, cl, a, rows, warps)) { clog[q] = cl; qapw[q] = a; break; }
         if (clog[q] < 0) return HAC_EUNSUPPORTED;
     }
     const int apws[5] = {2, 4, 8, 16, 32};
