@@ -116,8 +116,11 @@ def dist_env():
 # workload under profiles/ gives the command.  Reported as roofline.traffic
 # only for the same workload and layout: the per-instance layout
 # (ants_per_warp 0) with lookup lists, smallest cluster 1.
+# NCU_TRAFFIC is the capture of the warp-segment kernel, kept for comparison;
+# FUSED_TRAFFIC is the same capture of the present one (one ant per lane quad).
 _T_PER_INSTANCE = (0.613120768e9 + 0.943468032e9) + (6.650183680e9 + 3.744521984e9)
 NCU_TRAFFIC = {("batch128", 1, 0, 32, 0, 200): _T_PER_INSTANCE}
+FUSED_TRAFFIC = {("batch128", 1, 0, 32, 0, 200): (0.068993024e9 + 0.027493888e9) + (13.042279424e9 + 6.701411328e9)}
 
 
 def load_peaks():
@@ -662,7 +665,7 @@ def run_ours(args):
             "roofline": {"bound": "hbm", "kernel": kernel_name, "achieved": achieved,
                          "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                          "peak_kind": f"{peak_kind} HBM copy bandwidth",
-                         "traffic": NCU_TRAFFIC.get((args.workload, args.fused, ex.ants_per_warp, args.fbl,
+                         "traffic": FUSED_TRAFFIC.get((args.workload, args.fused, ex.ants_per_warp, args.fbl,
                                                      args.clog, ps[0].iterations)) if count == 128 else None,
                          "algorithmic_bytes_per_launch": per_launch_bytes,
                          "avg_launch_ms": avg_ms, "share_of_step": construct_share},
