@@ -1,7 +1,7 @@
 // One ant per lane (32 ants per warp): Algorithm 2 with the whole candidate
 // row of the current node in the lane's registers.
 //
-// The arithmetic is exactly that of the warp-segment construction (ant.cuh):
+// The arithmetic is exactly that of the lane-quad construction (ant_quad.cuh):
 // the k_pad slots form groups of 4 with sequential in-group partial sums, the
 // 8 group totals are combined by the same inclusive Hillis-Steele pattern
 // (offsets 1, 2, 4; zero totals beyond k_pad/4), slot prefixes are the

@@ -3,8 +3,8 @@
 //
 // Lane h (0 or 1) of a pair holds the slot groups g = 2j + h (j < NGL) of the
 // row: 4 consecutive slots per group, one vector load of ids and one of
-// choice values each.  The arithmetic is exactly that of the warp-segment
-// construction (ant.cuh) and of the oracle:
+// choice values each.  The arithmetic is exactly that of the lane-quad
+// construction (ant_quad.cuh) and of the oracle:
 //   - in-group partial sums, sequential over the group's 4 slots;
 //   - the group totals are swapped between the two lanes (one shuffle per
 //     group pair), so both lanes hold all of them, and the inclusive
@@ -17,14 +17,13 @@
 // Each lane finds the first qualifying slot among its own groups; one
 // shuffle between the lanes gives the pair's first slot and its node.
 //
-// Compared with 8-lane segments this takes one shuffle round instead of four
-// per step, and 16 instead of 4 ants share each warp instruction, so a warp
-// spends about a quarter of the instructions per ant-step.
+// Twice the ants of the lane quads share each warp instruction, but a lane
+// handles 12 slots alone and a warp waits for 16 ants' nearest-unvisited steps.
 //
 // The visited mask of pair p is stored word-major, pair-minor (word w at
 // w*16 + p): the 16 pairs of a warp use disjoint banks.  Lane 0 of the pair
 // sets the bits.  Nearest-unvisited steps (no live candidate) are served by
-// the whole warp, one pair after the other, as in ant.cuh.  Tours are written
+// the whole warp, one pair after the other, list, second list, scan.  Tours are written
 // ant-major, one entry per step, with the chosen slot (0xff for a
 // nearest-unvisited step); lengths are summed afterwards (lengths.cuh).
 #pragma once

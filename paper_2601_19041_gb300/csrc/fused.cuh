@@ -7,7 +7,7 @@
 // i in CTA i mod C).  Every construction step reads its row from local shared
 // memory or, through the cluster's distributed shared memory, from a
 // neighbouring SM, instead of from L2.  The ants are split over the CTAs, each
-// ant being a warp segment (ant.cuh).  Per iteration:
+// ant being a lane quad, pair or lane (ant_quad.cuh, ant_pair.cuh, ant_lane.cuh).  Per iteration:
 //   construct (all CTAs) -> cluster barrier ->
 //   iteration best, optional 2-opt of T_ib, global best, bounds, succ/pred
 //   (CTA 0) -> cluster barrier ->
