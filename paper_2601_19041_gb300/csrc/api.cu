@@ -110,7 +110,7 @@ static int plan_fused(hac_batch *bt, std::vector<int32_t> &order)
         return HAC_EUNSUPPORTED;            // the fused kernel has no 1-ant-per-warp form
     std::vector<int> members(bt->count);
     for (int b = 0; b < bt->count; ++b) members[b] = b;
-    return plan_groups(bt->zs, members, apw, bt->ex.cluster_log2, bt->ex.fallback_list, bt->groups, order);
+    return plan_groups(bt->zs, members, apw, bt->ex.cluster_log2, bt->ex.fallback_list, device_shape(), bt->groups, order);
 }
 
 // Everything hac_batch_create does after allocating the handle; on failure
@@ -188,7 +188,7 @@ static int batch_setup(hac_batch *bt, const hac_instance *ins, const hac_params 
     std::vector<int4> warpmap;
     long long ants = 0;
     for (const Sizes &z : P.zs) ants += z.m;
-    const int apw = bt->ex.ants_per_warp ? bt->ex.ants_per_warp : step_ants_per_warp(ants);   // per-step path (also the fallback)
+    const int apw = bt->ex.ants_per_warp ? bt->ex.ants_per_warp : step_ants_per_warp(ants, device_sms());   // per-step path (also the fallback)
     if (!bt->ex.fused) bt->ex.ants_per_warp = apw;
     for (BatchPart &pt : bt->parts) {
         pt.warp_off = (int)warpmap.size();

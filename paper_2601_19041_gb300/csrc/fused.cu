@@ -11,6 +11,45 @@ cudaError_t launch_fused_quad(const FusedArgs &A, const FusedLaunch &L)
     return launch_fused_form<8, 8, false>(A, L);
 }
 
+// a CTA that leaves room for no other on its SM, for device_shape
+__global__ void k_whole_sm() {}
+
+int device_sms()
+{
+    int d = 0, v = 0;
+    if (cudaGetDevice(&d) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, d) != cudaSuccess || v < 1) {
+        cudaGetLastError();
+        return DeviceShape().sms;
+    }
+    return v;
+}
+
+DeviceShape device_shape()
+{
+    DeviceShape S;
+    S.sms = S.clusters[0] = device_sms();
+    bool ok = cudaFuncSetAttribute(k_whole_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM_LIMIT) ==
+              cudaSuccess;
+    for (int c = 1; c <= 3 && ok; ++c) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 1u << c;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)S.sms << c, 1, 1);
+        cfg.blockDim = dim3(512, 1, 1);
+        cfg.dynamicSmemBytes = FUSED_SMEM_LIMIT;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int v = 0;
+        ok = cudaOccupancyMaxActiveClusters(&v, k_whole_sm, &cfg) == cudaSuccess;
+        if (ok && v > 0) S.clusters[c] = v;
+    }
+    if (!ok) cudaGetLastError();
+    return S;
+}
+
 size_t fused_smem_bytes(int rows_cap, int kp_cap, int warps, int apw, int stride, int xy_cap,
                         int list_rows)
 {

@@ -265,6 +265,15 @@ struct TailNeeds {
 };
 int launch_iteration_tail(const DevInst *d_inst, int count, const int2 *d_slotmap, int slotmap_len,
                           const TailNeeds &needs, int max_n, cudaStream_t s);
+// What the device takes at once, one CTA per SM: its SMs, and the clusters of
+// 2^c CTAs (fewer CTAs than SMs: a cluster lies within one GPC, so 152 SMs hold
+// 76 clusters of 2, 36 of 4 and 15 of 8).
+struct DeviceShape {
+    int sms = 152;
+    int clusters[4] = {152, 76, 36, 15};
+};
+int device_sms();                // of the current device
+DeviceShape device_shape();
 // fused cluster kernel (fused.cuh, fused.cu): one cluster of 2^clog CTAs per instance;
 // d_iters (parallel to d_order, may be null) gives each cluster its own
 // iteration count instead of `iters`
@@ -274,5 +283,6 @@ cudaError_t launch_fused(const DevInst *d_inst, const int32_t *d_order, const in
                          int clusters, int clog, int apw, bool ls, int warps, int block_warps, int rows_cap, int kp_cap,
                          int stride, int xy_cap, int list_rows, int iters, cudaStream_t s, bool after_resident);
 constexpr size_t FUSED_SMEM_LIMIT = 226 * 1024;   // dynamic shared memory per CTA we allow
+constexpr size_t SM_SMEM = 228 * 1024, CTA_SMEM_RESERVED = 1024;   // of an SM; taken by each CTA besides its own
 
 }  // namespace hac

@@ -30,7 +30,6 @@ constexpr int ROWS_PER_BLOCK = 8;      // matches the row kernels (8 warps, a ro
 constexpr int SLOTS_PER_BLOCK = 1024;  // matches the slot kernels
 constexpr int GRAPH_CHUNK = 10;        // iterations per captured graph
 constexpr int FBL_LEN = FBL1_LEN;      // nearest-unvisited lookup list
-constexpr int GPU_SMS = 152;           // SMs of a GB300
 
 // Ants per warp of the per-step kernels when the caller leaves it open: as few
 // as keep about 8 warps on every SM.  A warp's ants wait for each other's
@@ -38,9 +37,9 @@ constexpr int GPU_SMS = 152;           // SMs of a GB300
 // slots (16 x n = 5000, k = 20, 20 iterations end to end: 66.9 / 66.8 / 73.5 /
 // 83.9 ms with 1 / 2 / 4 / 8 ants per warp; one n = 500 instance, 100
 // iterations: 24.7 / 24.5 / 26.4 / 31.3 ms).
-inline int step_ants_per_warp(long long ants)
+inline int step_ants_per_warp(long long ants, int sms)
 {
-    const long long a = (ants + 8 * GPU_SMS - 1) / (8 * GPU_SMS);
+    const long long a = (ants + 8 * sms - 1) / (8 * sms);
     return a < 1 ? 1 : a > 8 ? 8 : (int)a;
 }
 
@@ -384,7 +383,7 @@ inline int upload_inputs(const DevInst &D, const hac_instance &in, const Sizes &
 // warp on one SM and in 275 ms with 4 ants per warp on the clusters.
 // `order` lists instance indices group after group.
 inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &members, int apw,
-                       int clog_min, int fallback_list, std::vector<FusedGroup> &groups,
+                       int clog_min, int fallback_list, const DeviceShape &dev, std::vector<FusedGroup> &groups,
                        std::vector<int32_t> &order)
 {
     const int count = (int)members.size();
@@ -448,10 +447,6 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
                     G.warps = std::max(G.warps, warps);
                 }
                 if (!G.count) continue;
-                // the warps beyond those that build tours share the rest of an
-                // iteration; 16 fill the SM's registers, so a group with more
-                // CTAs than SMs takes 8 and lets two CTAs share an SM
-                G.block_warps = std::max(G.warps, a > 8 ? 1 : (G.count << cl) > GPU_SMS ? 8 : 16);
                 const size_t base = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, 0, 0);
                 if (base > FUSED_SMEM_LIMIT) {
                     if (cl == 3) return HAC_EUNSUPPORTED;
@@ -472,6 +467,21 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
                 groups.push_back(G);
             }
         if (!again) break;
+    }
+    // Block width.  The warps beyond those that build tours share the rest of an
+    // iteration; 16 fill an SM's registers, so when the batch's CTAs -- all
+    // groups together, they run side by side -- outnumber what the device takes
+    // one to an SM, a CTA takes 8, 5 or 4 and lets 2, 3 or 4 share an SM, where
+    // their shared memory does (128 x n = 1000, m = 64 per iteration: on clusters of 8
+    // 2.09 ms with 8 warps a CTA and 1.13 with 4; 256 x n = 1000 on one SM each, no
+    // room for two: 1.31 ms with 8, 1.22 with 16).
+    double load = 0.0;
+    for (const FusedGroup &G : groups) load += (double)G.count / dev.clusters[G.clog];
+    for (FusedGroup &G : groups) {
+        const size_t smem = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, G.apw, G.stride, G.xy_cap, G.list_rows);
+        const int room = (int)(SM_SMEM / (smem + CTA_SMEM_RESERVED));
+        const int share = std::max(1, std::min(std::min((int)std::ceil(load), room), 4));
+        G.block_warps = std::max(G.warps, G.apw > 8 ? 1 : 16 / share);
     }
     // groups in order of their largest instance's work: the group launched
     // first gets SMs first, and the largest instances bound the batch

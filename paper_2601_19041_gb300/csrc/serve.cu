@@ -96,6 +96,7 @@ Region region_of(const Sizes &z)
 struct hac_server {
     hac_server_cfg cfg{};
     hac_exec ex{};
+    DeviceShape shape;
     cudaStream_t stream = nullptr;
     cudaStream_t prep[PREP_STREAMS] = {};
     int next_prep = 0;
@@ -176,7 +177,7 @@ int fits_fused(const hac_server *sv, const Sizes &z)
     std::vector<int> mem{0};
     std::vector<FusedGroup> g;
     std::vector<int32_t> o;
-    return plan_groups(one, mem, sv->ex.ants_per_warp, sv->ex.cluster_log2, sv->ex.fallback_list, g, o);
+    return plan_groups(one, mem, sv->ex.ants_per_warp, sv->ex.cluster_log2, sv->ex.fallback_list, sv->shape, g, o);
 }
 
 // per-tick tables of the per-step route: warp and slot work items
@@ -370,6 +371,7 @@ int hac_server_create(const hac_server_cfg *cfg, void *workspace, size_t ws_byte
     if (!sv) return HAC_ENOMEM;
     sv->cfg = c;
     sv->ex = ex;
+    sv->shape = device_shape();
     sv->stream = (cudaStream_t)stream;
     char *B = (char *)(((uintptr_t)workspace + 255) & ~(uintptr_t)255);
     Arena A;
@@ -539,7 +541,7 @@ int hac_server_tick(hac_server *sv)
         int32_t *h_ord = sv->h_order[par], *h_it = sv->h_order[par] + sv->cfg.max_slots;
         const size_t cnt = members.size();
         const bool together = plan_groups(sv->zs, members, sv->ex.ants_per_warp, sv->ex.cluster_log2,
-                                          sv->ex.fallback_list, groups, order) == HAC_OK;
+                                          sv->ex.fallback_list, sv->shape, groups, order) == HAC_OK;
         if (together) std::copy(order.begin(), order.end(), h_ord);
         else std::copy(members.begin(), members.end(), h_ord);
         for (size_t r = 0; r < cnt; ++r) h_it[r] = tick_iters(sv, sv->slots[h_ord[r]]);
@@ -553,7 +555,7 @@ int hac_server_tick(hac_server *sv)
             for (size_t r = 0; r < cnt; ++r) {
                 std::vector<int> one{h_ord[r]};
                 int st = plan_groups(sv->zs, one, sv->ex.ants_per_warp, sv->ex.cluster_log2,
-                                     sv->ex.fallback_list, groups, order);
+                                     sv->ex.fallback_list, sv->shape, groups, order);
                 if (st) return st;
                 if ((st = enqueue_groups(sv, groups, d_order + r, d_iters + r))) return st;
             }

@@ -1,0 +1,84 @@
+"""The layout of a batch in the cluster kernel (plan_groups, csrc/host.h), without
+a GPU: a small program made with the library's own header prints the groups of
+given batches on a device of 152 SMs that holds 76, 36 and 15 clusters of 2, 4
+and 8 CTAs."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+PROGRAM = r"""
+#include <cstdio>
+#include "host.h"
+using namespace hac;
+using namespace hac::host;
+// stdin: one batch a line: ants_per_warp cluster_log2 {count n m k local_search}...
+int main()
+{
+    char line[4096];
+    while (std::fgets(line, sizeof line, stdin)) {
+        int apw, clog, used, off = 0, c, n, m, k, ls;
+        if (std::sscanf(line, "%d %d%n", &apw, &clog, &off) != 2) continue;
+        std::vector<Sizes> zs;
+        while (std::sscanf(line + off, "%d %d %d %d %d%n", &c, &n, &m, &k, &ls, &used) == 5) {
+            Sizes z{};
+            z.n = n; z.m = m; z.kp = 4 * ((k + 3) / 4); z.k_eff = k; z.iters = 10; z.ls = ls;
+            zs.insert(zs.end(), c, z);
+            off += used;
+        }
+        std::vector<int> mem(zs.size());
+        for (size_t q = 0; q < mem.size(); ++q) mem[q] = (int)q;
+        std::vector<FusedGroup> g;
+        std::vector<int32_t> order;
+        const int st = plan_groups(zs, mem, apw, clog, 32, DeviceShape(), g, order);
+        std::printf("%d", st);
+        for (const FusedGroup &G : g)
+            std::printf(" %d,%d,%d,%d,%d,%zu", G.count, G.clog, G.apw, G.warps, G.block_warps,
+                        fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, G.apw, G.stride, G.xy_cap, G.list_rows));
+        std::printf("\n");
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    """plan(apw, clog, [(count, n, m, k, ls), ...]) -> status, [(count, clog, apw, warps, block_warps, smem), ...]"""
+    from paper_2601_19041_gb300 import build as B
+    cc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(cc):
+        pytest.skip("no nvcc")
+    lib = B.build()
+    d = tmp_path_factory.mktemp("plan")
+    src, exe = d / "plan.cu", d / "plan"
+    src.write_text(PROGRAM)
+    subprocess.run([cc, *B.ARCH, "-O1", "-std=c++17", "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include"),
+                    "-I", B.CSRC, str(src), "-o", str(exe), lib, "-Xlinker", f"-rpath={os.path.dirname(lib)}"], check=True)
+
+    def call(apw, clog, parts):
+        text = " ".join(map(str, [apw, clog] + [x for p in parts for x in p])) + "\n"
+        out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True).stdout.split()
+        return int(out[0]), [tuple(int(v) for v in g.split(",")) for g in out[1:]]
+    return call
+
+
+# An SM holds 16 warps of the cluster kernel and 228 KB of shared memory.
+@pytest.mark.parametrize("apw,clog,parts,block", [
+    (0, 0, [(128, 500, 32, 20, 0)], 16),                             # an SM each
+    (0, 0, [(256, 500, 32, 20, 0)], 8),                              # two share an SM
+    (0, 0, [(256, 1000, 64, 20, 0)], 16),                            # too large to share one
+    (0, 0, [(100, 500, 32, 20, 0), (100, 500, 32, 20, 1)], 8),       # two groups side by side
+    (0, 1, [(76, 500, 32, 20, 0)], 16),
+    (0, 2, [(36, 1000, 64, 20, 0)], 16),
+    (0, 3, [(16, 1000, 64, 20, 0)], 8),                              # 15 clusters of 8 fit
+    (2, 3, [(128, 500, 32, 20, 0)], 4),
+])
+def test_block_width(plan, apw, clog, parts, block):
+    st, groups = plan(apw, clog, parts)
+    assert st == 0 and sum(g[0] for g in groups) == sum(p[0] for p in parts)
+    for count, cl, a, warps, bw, smem in groups:
+        assert bw == max(block, warps), groups
+        assert smem <= 226 * 1024
