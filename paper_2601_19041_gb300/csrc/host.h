@@ -375,9 +375,9 @@ inline int upload_inputs(const DevInst &D, const hac_instance &in, const Sizes &
 // Groups the given instances by layout: local search or none, ants per warp and cluster size (the
 // fewest CTAs whose shared memory holds the instance's share of the
 // candidate table and visited masks, at least 2^clog_min), each group ordered
-// by decreasing work.  apw = 0 stands for 8 ants per warp, on one CTA where the
-// instance fits one with its coordinates, else on the smallest cluster that
-// holds it.  8 ants per warp keep the fewest warps waiting for issue slots: 64
+// by decreasing work.  apw = 0 stands for 8 ants per warp on one CTA where the
+// instance fits one with its coordinates, else for the smallest cluster that
+// holds it and as many ants per warp as its CTAs need (below).  8 ants per warp keep the fewest warps waiting for issue slots: 64
 // ants on one SM take 839 cycles per step at n = 500 on 8 warps and 1127 on 16;
 // 128 instances of n ~ U{500..2000} decode in 250 ms, in 263 ms with 4 ants per
 // warp on one SM and in 275 ms with 4 ants per warp on the clusters.
@@ -420,6 +420,26 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
             for (int cl = clog_min; cl <= 3; ++cl)
                 if (fits(q, cl, a, rows, warps)) { clog[q] = cl; qapw[q] = a; break; }
         if (clog[q] < 0) return HAC_EUNSUPPORTED;
+    }
+    if (apw == 0) {
+        // Ants per warp on a cluster: as few as keep 8 warps on an SM, as on the
+        // per-step path -- a warp's ants wait for each other's nearest-unvisited
+        // steps (per iteration, with 8 ants per warp / with this rule: 32 x n = 6000,
+        // k = 10, m = 32 on 2 CTAs 4.38 / 2.94 ms; 128 x n = 4000, m = 64 on 4 9.13 /
+        // 7.60; 16 x n = 1000, m = 64 on 8 1.00 / 0.46).
+        double load = 0.0;
+        for (int q = 0; q < count; ++q) load += 1.0 / dev.clusters[clog[q]];
+        for (int q = 0; q < count; ++q) {
+            if (clog[q] == 0) continue;
+            const Sizes &z = zs[members[q]];
+            for (int a = 2; a < qapw[q]; a *= 2) {
+                int rows, warps;
+                if (!fits(q, clog[q], a, rows, warps)) continue;
+                const size_t smem = fused_smem_bytes(rows, z.kp, warps, a, (z.n + 32) / 32, z.n, 0);
+                const int share = std::max(1, std::min((int)std::ceil(load), (int)(SM_SMEM / (smem + CTA_SMEM_RESERVED))));
+                if (share * warps <= 8) { qapw[q] = a; break; }
+            }
+        }
     }
     const int apws[5] = {2, 4, 8, 16, 32};
     auto in_group = [&](int q, int cl, int a, int ls) {

@@ -82,3 +82,20 @@ def test_block_width(plan, apw, clog, parts, block):
     for count, cl, a, warps, bw, smem in groups:
         assert bw == max(block, warps), groups
         assert smem <= 226 * 1024
+
+
+# On a cluster, as few ants per warp (2, 4, 8) as leave at most 8 warps on an SM.
+@pytest.mark.parametrize("clog,part,apw", [
+    (3, (8, 1000, 64, 20, 0), 2),        # 8 ants per CTA
+    (2, (32, 1000, 64, 20, 0), 2),       # 16
+    (1, (32, 1000, 64, 20, 0), 4),       # 32
+    (1, (32, 1000, 128, 20, 0), 8),      # 64
+    (1, (128, 1000, 64, 20, 0), 8),      # 32, two CTAs to an SM
+    (0, (32, 6000, 32, 10, 0), 2),       # too large for one SM: 2 CTAs
+    (0, (128, 4000, 64, 20, 0), 2),      # 4 CTAs, room for one on an SM
+    (0, (128, 2000, 64, 20, 0), 4),      # 2 CTAs
+    (0, (128, 1000, 64, 20, 0), 8),      # one SM
+])
+def test_ants_per_warp_on_clusters(plan, clog, part, apw):
+    st, groups = plan(0, clog, [part])
+    assert st == 0 and [(g[0], g[2]) for g in groups] == [(part[0], apw)], groups
