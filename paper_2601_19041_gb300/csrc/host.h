@@ -422,6 +422,26 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
         if (clog[q] < 0) return HAC_EUNSUPPORTED;
     }
     if (apw == 0) {
+        // More than 64 ants on one SM are more than 8 warps, which wait for issue
+        // slots, and on a cluster more than 32 per CTA leave 8 to a warp: while SMs
+        // are idle, these instances go to the largest cluster of which the device
+        // takes all at once (per iteration, without / with this rule: 8 x n = 500,
+        // m = 100 0.364 / 0.239 ms; 32 x n = 1000, m = 96 0.714 / 0.527; 64 x n = 1000,
+        // m = 100 0.851 / 0.631; 32 x n = 2000, m = 128 1.44 / 1.06).
+        int crowded = 0, other = 0;
+        auto crowds = [&](int q) { return (zs[members[q]].m - 1) >> clog[q] >= (clog[q] ? 32 : 64); };
+        for (int q = 0; q < count; ++q) {
+            if (crowds(q)) ++crowded;
+            else other += 1 << clog[q];
+        }
+        for (int cl = 3; cl >= 1 && crowded; --cl) {
+            if (crowded > dev.clusters[cl] || (crowded << cl) + other > dev.sms) continue;
+            for (int q = 0; q < count; ++q) {
+                int rows, warps;
+                if (clog[q] < cl && crowds(q) && fits(q, cl, 8, rows, warps)) { clog[q] = cl; qapw[q] = 8; }
+            }
+            break;
+        }
         // Ants per warp on a cluster: as few as keep 8 warps on an SM, as on the
         // per-step path -- a warp's ants wait for each other's nearest-unvisited
         // steps (per iteration, with 8 ants per warp / with this rule: 32 x n = 6000,

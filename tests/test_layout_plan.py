@@ -89,7 +89,7 @@ def test_block_width(plan, apw, clog, parts, block):
     (3, (8, 1000, 64, 20, 0), 2),        # 8 ants per CTA
     (2, (32, 1000, 64, 20, 0), 2),       # 16
     (1, (32, 1000, 64, 20, 0), 4),       # 32
-    (1, (32, 1000, 128, 20, 0), 8),      # 64
+    (1, (60, 1000, 128, 20, 0), 8),      # 64
     (1, (128, 1000, 64, 20, 0), 8),      # 32, two CTAs to an SM
     (0, (32, 6000, 32, 10, 0), 2),       # too large for one SM: 2 CTAs
     (0, (128, 4000, 64, 20, 0), 2),      # 4 CTAs, room for one on an SM
@@ -99,3 +99,17 @@ def test_block_width(plan, apw, clog, parts, block):
 def test_ants_per_warp_on_clusters(plan, clog, part, apw):
     st, groups = plan(0, clog, [part])
     assert st == 0 and [(g[0], g[2]) for g in groups] == [(part[0], apw)], groups
+
+
+# More than 64 ants on one SM, or more than 32 on a CTA of a cluster: the largest
+# cluster of which all fit on the device at once.
+@pytest.mark.parametrize("parts,clogs", [
+    ([(15, 500, 128, 20, 0)], [3]), ([(16, 500, 128, 20, 0)], [2]), ([(36, 500, 65, 20, 0)], [2]),
+    ([(37, 500, 65, 20, 0)], [1]), ([(76, 500, 65, 20, 0)], [1]), ([(77, 500, 65, 20, 0)], [0]),
+    ([(1, 500, 64, 20, 0)], [0]), ([(1, 500, 1000, 20, 0)], [3]), ([(1, 500, 256, 20, 0)], [3]),
+    ([(32, 2000, 64, 20, 0)], [1]), ([(32, 2000, 65, 20, 0)], [2]), ([(37, 2000, 128, 20, 0)], [1]),
+    ([(10, 500, 100, 20, 0), (80, 500, 32, 20, 0)], [0, 2]), ([(10, 500, 100, 20, 0), (140, 500, 32, 20, 0)], [0]),
+])
+def test_crowded_instances_spread_over_idle_sms(plan, parts, clogs):
+    st, groups = plan(0, 0, parts)
+    assert st == 0 and sorted(set(g[1] for g in groups)) == clogs, groups
