@@ -64,7 +64,7 @@ cudaError_t launch_fused(const DevInst *d_inst, const int32_t *d_order, const in
     const FusedArgs A{d_inst, d_order, d_iters, iters, rows_cap, kp_cap, stride, warps, apw, xy_cap, list_rows};
     const FusedLaunch L{clog, clusters, block_warps,
                         fused_smem_bytes(rows_cap, kp_cap, warps, apw, stride, xy_cap, list_rows), s, after_resident};
-    if (apw > 8) return launch_fused_lane(A, L);
+    if (apw > 8) return ls ? launch_fused_lane_ls(A, L) : launch_fused_lane(A, L);
     return ls ? launch_fused_quad_ls(A, L) : launch_fused_quad(A, L);
 }
 

@@ -76,7 +76,8 @@ __host__ __device__ inline size_t fused_vis_bytes(int warps, int apw, int stride
 // LS: the group's instances may use local search.  Without it the kernel holds
 // no call, and the construction loop gets the registers: 128 instances of n ~
 // U{500..2000} take 241 ms without the searches' code in the kernel and
-// 336 ms with it (end to end, 200 iterations).
+// 336 ms with it (end to end, 200 iterations).  With one ant per lane pair,
+// 128 x n = 1000, m = 64 on 2 CTAs take 1.28 ms per iteration without, 1.89 with it.
 template <int APW, int NG, int CLOG, bool LS>
 __global__ void __launch_bounds__(512, 1) k_fused(FusedArgs A)
 {
@@ -303,5 +304,6 @@ inline cudaError_t launch_fused_form(const FusedArgs &A, const FusedLaunch &L)
 cudaError_t launch_fused_quad(const FusedArgs &A, const FusedLaunch &L);      // fused.cu
 cudaError_t launch_fused_quad_ls(const FusedArgs &A, const FusedLaunch &L);   // fused_ls.cu
 cudaError_t launch_fused_lane(const FusedArgs &A, const FusedLaunch &L);      // fused_lane.cu
+cudaError_t launch_fused_lane_ls(const FusedArgs &A, const FusedLaunch &L);   // fused_lane_ls.cu
 
 }  // namespace hac

@@ -49,3 +49,11 @@ def test_many_ants(hac, orc, n, m, count):
 @pytest.mark.parametrize("clog,m,count", [(1, 16, 3), (1, 30, 160), (2, 33, 80), (3, 9, 40), (3, 64, 16), (3, 5, 130)])
 def test_clusters(hac, orc, clog, m, count):
     _check(hac, orc, *_instances(70, m, count, k=29), hac.make_exec(fused=1, fallback_list=32, cluster_log2=clog))
+
+
+@pytest.mark.parametrize("apw", [0, 2, 4, 16, 32])
+@pytest.mark.parametrize("clog", [0, 1])
+def test_groups_with_and_without_local_search(hac, orc, apw, clog):
+    ins, ps = _instances(90, 20, 4)
+    ins2, ps2 = _instances(61, 9, 4, local_search=1, ls_k=8)
+    _check(hac, orc, ins + ins2, ps + ps2, hac.make_exec(apw, fused=1, fallback_list=32, cluster_log2=clog))
