@@ -135,10 +135,11 @@ typedef struct {
 /* Execution options of a batch (none of them changes any result). */
 typedef struct {
     int32_t ants_per_warp;    /* 1, 2 or 4 ants share one warp (a lane quad each), 16 (one ant per
-                                 lane pair) or 32 (one ant per lane); 0 = auto (fused: 8,
+                                 lane pair) or 32 (one ant per lane); 0 = auto (fused: 8
                                  on one CTA when the instance's table, visited masks and
-                                 coordinates fit in one SM's shared memory, else on a cluster;
-                                 per-step: as few as keep about 8 warps on every SM) */
+                                 coordinates fit in one SM's shared memory, else 2, 4 or 8 on a
+                                 cluster, where instances of more than 64 ants also go while SMs
+                                 are idle; per-step: as few as keep about 8 warps on every SM) */
     int32_t warps_per_block;  /* construction block size in warps; 0 = auto */
     int32_t use_graph;        /* 1: capture the iteration loop (per-step kernels: 10 iterations
                                  per graph; fused: the group launches) in a CUDA
@@ -259,10 +260,9 @@ int hac_batch_kernel_time(hac_batch *bt, int32_t group, double *ms, int64_t *lau
  * ants per warp or the per-instance choice (0), smallest cluster 1, 2 or 4
  * CTAs, with and without the 32-entry nearest-unvisited lookup list; the
  * per-step kernels with 1, 2, 4 or 16 ants per warp and 4 or 8 warps per
- * block.  The per-instance choice is returned when it is at least 2 % faster
- * than every other candidate.  No layout changes a result, so the choice
- * is a matter of speed only; the method's parameters (m, k, ...) are never
- * changed.  Uses `workspace` (hac_batch_workspace_size bytes) for each trial
+ * block, and with the ants per warp (and the block) left open.  No layout
+ * changes a result, so the choice is a matter of speed only; the method's
+ * parameters (m, k, ...) are never changed.  Uses `workspace` (hac_batch_workspace_size bytes) for each trial
  * in turn; synchronises `stream`.  Candidates an instance does not support
  * are skipped. */
 int hac_batch_autotune(const hac_instance *ins, const hac_params *ps, int32_t count,

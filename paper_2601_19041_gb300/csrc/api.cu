@@ -695,81 +695,48 @@ int hac_batch_autotune(const hac_instance *ins, const hac_params *ps, int32_t co
     int st = plan_batch(ins, ps, count, inputs_on_device, P);
     if (st) return st;
     if (!workspace || ws_bytes < P.total) return HAC_ENOMEM;
-    // candidates: every execution layout (none changes a result)
-    std::vector<hac_exec> cands;
-    for (int apw : {0, 16, 4, 2, 32})
-        for (int clog = 0; clog <= 2; ++clog)
-            for (int fbl : {FBL_LEN, 0}) {
-                hac_exec e;
-                hac_exec_default(&e);
-                e.fused = 1; e.ants_per_warp = apw; e.cluster_log2 = clog; e.fallback_list = fbl;
-                cands.push_back(e);
-            }
-    for (int apw : {16, 4, 2, 1})
-        for (int wpb : {4, 8})
-            for (int parts : {1, 4}) {
-                if (parts > count) continue;
-                hac_exec e;
-                hac_exec_default(&e);
-                e.fused = 0; e.ants_per_warp = apw; e.warps_per_block = wpb; e.fallback_list = FBL_LEN;
-                e.parts = parts;
-                cands.push_back(e);
-            }
+    long long ants = 0;
+    for (const Sizes &z : P.zs) ants += z.m;
+    const std::vector<hac_exec> cands = tune_candidates(count, step_ants_per_warp(ants, device_sms()));
     cudaStream_t s = (cudaStream_t)stream;
     cudaEvent_t ev[2];
     CK(cudaEventCreate(&ev[0]));
     if (cudaEventCreate(&ev[1]) != cudaSuccess) { cudaEventDestroy(ev[0]); return HAC_ECUDA; }
-    // one trial of layout c: its time for trial_iters iterations, -1 when an
-    // instance does not support it (or the layout is a per-step one in disguise)
-    auto trial = [&](const hac_exec &c, float &ms) {
+    double best_ms = -1.0;
+    hac_exec pick{};
+    int rc = HAC_OK;
+    for (const hac_exec &c : cands) {
         hac_exec e = c;
         e.use_graph = 0;
-        ms = -1.f;
         hac_batch *bt = nullptr;
-        int st = hac_batch_create(ins, ps, count, inputs_on_device, workspace, ws_bytes, &e, stream, &bt);
-        if (st) return st == HAC_EUNSUPPORTED ? HAC_OK : st;
+        st = hac_batch_create(ins, ps, count, inputs_on_device, workspace, ws_bytes, &e, stream, &bt);
+        if (st == HAC_EUNSUPPORTED) continue;
+        if (st) { rc = st; break; }
         if (e.fused && !bt->ex.fused) {   // does not fit the cluster kernel: same as a per-step candidate
             hac_batch_destroy(bt);
-            return (int)HAC_OK;
+            continue;
         }
-        float t = 0.f;
+        float ms = 0.f;
         st = hac_batch_iterate(bt, 1);
         if (!st && cudaEventRecord(ev[0], s) != cudaSuccess) st = HAC_ECUDA;
         if (!st) st = hac_batch_iterate(bt, trial_iters);
         if (!st && cudaEventRecord(ev[1], s) != cudaSuccess) st = HAC_ECUDA;
         if (!st) st = hac_batch_sync(bt);
-        if (!st && cudaEventElapsedTime(&t, ev[0], ev[1]) != cudaSuccess) st = HAC_ECUDA;
+        if (!st && cudaEventElapsedTime(&ms, ev[0], ev[1]) != cudaSuccess) st = HAC_ECUDA;
         hac_batch_destroy(bt);
-        if (!st) ms = t;
-        return st;
-    };
-    // the best layout that names its ants per warp, and the best that leaves
-    // them to the library (0): on many batches the two take the same time
-    double best_ms[2] = {-1.0, -1.0};
-    hac_exec pick[2] = {};
-    int rc = HAC_OK;
-    for (const hac_exec &c : cands) {
-        float ms;
-        if ((rc = trial(c, ms))) break;
-        const int open = c.ants_per_warp == 0;
-        if (ms >= 0.f && (best_ms[open] < 0.0 || ms < best_ms[open])) { best_ms[open] = ms; pick[open] = c; }
-    }
-    // the open one has to be 2 % faster, also when both are timed again in turn
-    int w = best_ms[0] < 0.0 ? 1 : 0;
-    if (!rc && best_ms[1] >= 0.0 && best_ms[0] >= 0.0 && best_ms[1] < 0.98 * best_ms[0]) {
-        for (int q = 0; q < 4 && !rc; ++q) {
-            float ms;
-            if (!(rc = trial(pick[q & 1], ms)) && ms >= 0.f) best_ms[q & 1] = std::min(best_ms[q & 1], (double)ms);
+        if (st) { rc = st; break; }
+        if (best_ms < 0.0 || ms < best_ms) {
+            best_ms = ms;
+            pick = c;
         }
-        w = best_ms[1] < 0.98 * best_ms[0] ? 1 : 0;
     }
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
     if (rc) return rc;
-    if (best_ms[w] < 0.0) return HAC_EUNSUPPORTED;
-    *best = pick[w];
+    if (best_ms < 0.0) return HAC_EUNSUPPORTED;
+    *best = pick;
     best->use_graph = 1;
-    if (ms_per_iter) *ms_per_iter = best_ms[w] / trial_iters;
+    if (ms_per_iter) *ms_per_iter = best_ms / trial_iters;
     return HAC_OK;
 }
 

@@ -43,6 +43,26 @@ inline int step_ants_per_warp(long long ants, int sms)
     return a < 1 ? 1 : a > 8 ? 8 : (int)a;
 }
 
+// The autotuner's candidates for `count` instances: every execution layout of
+// the cluster kernel, then the per-step kernels; step_apw is what they take
+// when their ants per warp are left open, which is among them.
+inline std::vector<hac_exec> tune_candidates(int count, int step_apw)
+{
+    std::vector<hac_exec> c;
+    for (int apw : {0, 16, 4, 2, 32})
+        for (int clog = 0; clog <= 2; ++clog)
+            for (int fbl : {FBL_LEN, 0}) c.push_back(hac_exec{apw, 0, 1, 1, fbl, 0, clog, 0});
+    for (int parts : {1, 4}) {
+        if (parts > count) continue;
+        for (int apw : {16, 4, 2, 1, 0})
+            for (int wpb : {4, 8})   // left open only where it is none of the others
+                if (apw || (step_apw != 1 && step_apw != 2 && step_apw != 4))
+                    c.push_back(hac_exec{apw, wpb, 1, 0, FBL_LEN, 0, 0, parts});
+        c.push_back(hac_exec{0, 0, 1, 0, FBL_LEN, 0, 0, parts});
+    }
+    return c;
+}
+
 struct Arena {
     size_t off = 0;
     size_t take(size_t bytes)

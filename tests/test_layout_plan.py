@@ -12,12 +12,20 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 PROGRAM = r"""
 #include <cstdio>
+#include <cstdlib>
 #include "host.h"
 using namespace hac;
 using namespace hac::host;
 // stdin: one batch a line: ants_per_warp cluster_log2 {count n m k local_search}...
-int main()
+// with arguments count and step_apw: the autotuner's candidates instead
+int main(int argc, char **argv)
 {
+    if (argc == 3) {
+        for (const hac_exec &e : tune_candidates(std::atoi(argv[1]), std::atoi(argv[2])))
+            std::printf("%d,%d,%d,%d,%d,%d,%d,%d ", e.ants_per_warp, e.warps_per_block, e.use_graph, e.fused,
+                        e.fallback_list, e.profile, e.cluster_log2, e.parts);
+        return 0;
+    }
     char line[4096];
     while (std::fgets(line, sizeof line, stdin)) {
         int apw, clog, used, off = 0, c, n, m, k, ls;
@@ -58,7 +66,10 @@ def plan(tmp_path_factory):
     subprocess.run([cc, *B.ARCH, "-O1", "-std=c++17", "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include"),
                     "-I", B.CSRC, str(src), "-o", str(exe), lib, "-Xlinker", f"-rpath={os.path.dirname(lib)}"], check=True)
 
-    def call(apw, clog, parts):
+    def call(apw, clog, parts=None):
+        if parts is None:      # the autotuner's candidates for apw instances, clog ants per warp if left open
+            out = subprocess.run([str(exe), str(apw), str(clog)], capture_output=True, text=True, check=True).stdout
+            return [tuple(int(v) for v in c.split(",")) for c in out.split()]
         text = " ".join(map(str, [apw, clog] + [x for p in parts for x in p])) + "\n"
         out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True).stdout.split()
         return int(out[0]), [tuple(int(v) for v in g.split(",")) for g in out[1:]]
@@ -113,3 +124,22 @@ def test_ants_per_warp_on_clusters(plan, clog, part, apw):
 def test_crowded_instances_spread_over_idle_sms(plan, parts, clogs):
     st, groups = plan(0, 0, parts)
     assert st == 0 and sorted(set(g[1] for g in groups)) == clogs, groups
+
+
+# The tuner times what a per-step call with the layout left open runs, and only
+# layouts that a batch accepts.
+@pytest.mark.parametrize("count,step_apw", [(1, 1), (3, 2), (4, 4), (60, 3), (100, 6), (500, 8)])
+def test_autotuner_candidates(plan, count, step_apw):
+    cands = plan(count, step_apw)
+    assert len(set(cands)) == len(cands)
+    for parts in (1, 4):
+        mine = [c for c in cands if not c[3] and c[7] == parts]
+        if parts > count:
+            assert not mine
+            continue
+        assert (0, 0, 1, 0, 32, 0, 0, parts) in mine
+        for wpb in (4, 8):
+            assert ((0, wpb, 1, 0, 32, 0, 0, parts) in mine) == (step_apw not in (1, 2, 4))
+    for apw, wpb, graph, fused, fbl, prof, clog, parts in cands:
+        assert apw in (0, 1, 2, 4, 16, 32) and 0 <= wpb <= 8 and graph == 1 and fbl in (0, 32) and prof == 0
+        assert fused == 0 or (apw != 1 and 0 <= clog <= 3)
