@@ -331,10 +331,12 @@ __device__ void warp_knn(const DevInst &I, int i, int K, Pred pred, double &dout
     int nc = 0;
     bool ovf = false;
     // from the kept keys when every lane kept all of its nodes inside the margin
+    // (nodes whose key overflows are never kept: no margin may reach them)
     int within = 0;
 #pragma unroll
     for (int c = 0; c < KEEP; ++c) within += ru[c] != 0x7fffffff && rk[c] <= thr;
-    const bool kept = known && __all_sync(FULL, within <= CACHE && (seen_all <= KEEP || rk[KEEP - 1] > thr));
+    const bool kept = known && thr < __int_as_float(0x7f800000) &&
+                      __all_sync(FULL, within <= CACHE && (seen_all <= KEEP || rk[KEEP - 1] > thr));
     if (kept) {
 #pragma unroll
         for (int c = 0; c < CACHE; ++c) {
