@@ -52,7 +52,7 @@ enum hac_status {
     HAC_EBUSY = -6          /* serving: request not finished yet / no slot free */
 };
 
-#define HAC_KMAX 32         /* candidate-list size limit (one 8-lane warp segment) */
+#define HAC_KMAX 32         /* candidate-list size limit (8 groups of 4 slots) */
 #define HAC_NMAX (1 << 20)  /* node-count limit of one instance */
 #define HAC_MMAX 1024       /* ants per instance */
 

@@ -4,17 +4,17 @@
 // Lane h of a quad holds the slot groups 4j + h (j < NGL); with TAIL (five
 // groups, k <= 20) the fifth group is split, lane h holding its slot 16 + h,
 // so that 20 slots keep all four lanes busy.  The arithmetic is exactly that
-// of the warp-segment construction (ant.cuh) and of the oracle: sequential
-// in-group partial sums, the 8 group totals combined by the Hillis-Steele
-// pattern (GroupScan), slot prefix = exclusive group prefix + in-group sum,
-// r = fl32(u * total), the first live slot with r < prefix, or the last live
-// slot when rounding leaves none.
+// of the other forms (ant.cuh) and of the oracle: sequential in-group partial
+// sums, the 8 group totals combined by the Hillis-Steele pattern (GroupScan),
+// slot prefix = exclusive group prefix + in-group sum, r = fl32(u * total), the
+// first live slot with r < prefix, or the last live slot when rounding leaves
+// none.
 //
 // What bounds it: the dependent chain of a step (row load -> visited bits ->
 // in-group sums -> group totals -> prefix -> chosen node -> next row), about
 // 640 cycles with 4 warps on an SM (n = 500, m = 32, rows in shared memory), 840
 // with 8 (m = 64).  The layout this replaces spread an ant over 8 or 16 lanes
-// and took 1450 to 1580 cycles for 64 ants on 16 warps: the same chain, but
+// and took 1368 to 1580 cycles for 64 ants on 16 warps: the same chain, but
 // four times the warp instructions for it.  Four lanes are the fewest that
 // still load a row in one go; what shortened the chain besides:
 //   - no value or load hangs on a divergent branch (padding slots are a node
@@ -34,7 +34,7 @@
 // Nearest-unvisited steps (no live candidate): all quads that need one read
 // their node's 32-entry list at once, 8 entries per lane; what the list does
 // not answer is served by the whole warp, one ant after the other (second
-// list, then a scan), as in ant.cuh.
+// list, then a scan).
 #pragma once
 
 #include "ant.cuh"
@@ -403,7 +403,6 @@ __device__ __forceinline__ void build_tours_quad(const DevInst &I, const Rows &r
 #pragma unroll
                 for (int g = 0; g < GT; ++g) live |= T[g] > 0.0f;
                 const bool need = real & !live;
-                // the second list of the first ant that needs a node, in flight meanwhile
                 unsigned pend = __ballot_sync(FULL_MASK, need & (h == 0));
                 if (__any_sync(FULL_MASK, live & !hit)) {   // rounding left no r < prefix: the last live slot
                     int ll = -1, ln = 0;

@@ -1,7 +1,8 @@
 // Tour construction, Algorithm 2, one launch per iteration: every ant of every
 // active instance builds one tour, reading candidate rows from global memory
-// (128-bit loads of ids and choice values).  The per-ant work is build_tours
-// in ant.cuh; this file maps warps to (instance, ants) through the warp table.
+// (128-bit loads of ids and choice values).  The per-ant work is in ant_quad.cuh,
+// ant_pair.cuh and ant_lane.cuh; this file maps warps to (instance, ants)
+// through the warp table.
 #include "ant_lane.cuh"
 #include "ant_pair.cuh"
 #include "ant_quad.cuh"

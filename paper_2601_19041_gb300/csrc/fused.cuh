@@ -15,7 +15,7 @@
 //   shared memory (each CTA its own rows) -> cluster barrier.
 // Cluster barriers are hardware barriers (no spinning); all CTAs of a cluster
 // run the same number of iterations.  The arithmetic is exactly that of the
-// per-iteration kernels (ant.cuh, iter.cuh, twoopt.cuh).
+// per-iteration kernels (construct.cu, iter.cuh, twoopt.cuh).
 #pragma once
 
 #include <cooperative_groups.h>

@@ -584,7 +584,7 @@ __device__ __forceinline__ void ls_rounds(const LsMem &M, int n, Examine &&exami
 // Improves the ATSP `tour` (global memory) in place by the directed 2-opt.
 static __device__ __noinline__ void warp_two_opt_directed(const DevInst &I, int32_t *tour, const LsMem &Mref)
 {
-    const LsMem M = Mref;   // a local copy: see warp_two_opt
+    const LsMem M = Mref;   // a local copy: see warp_two_opt_body
     const int lane = threadIdx.x & 31;
     const int n = I.n, K = I.ls_k;
     if (M.tour != tour)
@@ -673,7 +673,7 @@ __device__ __forceinline__ void block_local_search(const DevInst &I, int32_t *to
 {
     const int warps = (int)(blockDim.x >> 5);
     if (I.kind == 1) {                 // directed: one warp, no helpers
-        if (threadIdx.x < 32) warp_two_opt_directed(I, tour, ls_shared(I, tour, sm, smem_bytes, ls_global(I, tour)));
+        if (threadIdx.x < 32) warp_two_opt_directed(I, tour, ls_shared(I, sm, smem_bytes, ls_global(I, tour)));
         __syncthreads();
     } else if (ls_smem_full(I.n) <= smem_bytes) {
         LsMem M = ls_shared_full(I, sm);
@@ -683,7 +683,7 @@ __device__ __forceinline__ void block_local_search(const DevInst &I, int32_t *to
         M.coop_warps = warps;
         block_search(I, tour, M);
     } else {
-        LsMem M = ls_shared(I, tour, sm, smem_bytes, ls_global(I, tour), false);
+        LsMem M = ls_shared(I, sm, smem_bytes, ls_global(I, tour));
         M.coop = coop;
         M.coop_warps = warps;
         block_search(I, tour, M);

@@ -54,7 +54,7 @@ __global__ void k_two_opt_all(const DevInst *insts, int max_m, unsigned smem_byt
         if (I.local_search == 4) warp_three_opt_body(I, tour, M);
         else warp_two_opt_body(I, tour, M);
     } else {
-        const LsMem M = ls_shared(I, tour, ls_sm, smem_bytes, ls_ant(I, a));
+        const LsMem M = ls_shared(I, ls_sm, smem_bytes, ls_ant(I, a));
         if (I.local_search == 4) warp_three_opt(I, tour, M);
         else warp_two_opt_any(I, tour, M);
     }

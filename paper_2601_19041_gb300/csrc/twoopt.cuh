@@ -1,6 +1,6 @@
 // First-improvement 2-opt with geometric neighbour lists and don't-look bits
-// (Sec. III-D), one warp per instance, applied to T_NN once (Algorithm 1's initialisation)
-// and to the iteration-best tour before it updates the pheromone.
+// (Sec. III-D), applied to T_NN once (Algorithm 1's initialisation) and to the
+// iteration-best tour or every ant's tour before they update the pheromone.
 //
 // Order of the search (it defines the result):
 //   rounds start with all bits clear; a round repeats passes over the tour
@@ -195,7 +195,7 @@ __device__ __forceinline__ void ls_reverse_part(const LsMem &M, int n, int i0, i
 // One pre-test work item: candidate move of city a in direction dir (0: succ,
 // 1: pred) with its q-th neighbour; true unless the FP64 gain is certainly
 // <= LS_GAIN.  an, da: the city's dir-neighbour and FP32 edge length.
-__device__ __forceinline__ bool ls_item_may_improve(const DevInst &I, const LsMem &M, int n, int K, int a, int dir,
+__device__ __forceinline__ bool ls_item_may_improve(const LsMem &M, int n, int K, int a, int dir,
                                                    int q, int an, float da)
 {
     const int b = M.nbr[(size_t)a * K + q];
@@ -521,8 +521,7 @@ __device__ __forceinline__ void ls2_apply(const LsMem &M, int n, const LsMove &F
 // items of all cities are dealt to the lanes in position order, 32 at a time;
 // after the first group with a possible move every earlier city has been
 // tested in full, so the search stops there.
-__device__ __forceinline__ int ls_first_may_move(const DevInst &I, const LsMem &M, int n, int K, bool clear, int al,
-                                                 int pp)
+__device__ __forceinline__ int ls_first_may_move(const LsMem &M, int n, int K, bool clear, int al, int pp)
 {
     const int lane = threadIdx.x & 31;
     int an0 = 0, an1 = 0, c0 = 0, c1 = 0;
@@ -571,7 +570,7 @@ __device__ __forceinline__ int ls_first_may_move(const DevInst &I, const LsMem &
         bool hit = false;
         if (t < total) {
             const int dir = j < cc0 ? 0 : 1;
-            hit = ls_item_may_improve(I, M, n, K, a, dir, dir == 0 ? j : j - cc0, dir == 0 ? xan0 : xan1,
+            hit = ls_item_may_improve(M, n, K, a, dir, dir == 0 ? j : j - cc0, dir == 0 ? xan0 : xan1,
                                       dir == 0 ? xda0 : xda1);
         }
         const unsigned first = __reduce_min_sync(FULL2, hit ? (unsigned)c : 32u);
@@ -672,7 +671,7 @@ __device__ __forceinline__ void warp_two_opt_body(const DevInst &I, int32_t *tou
                         ls_prefetch_row(M.nbrd32 + (size_t)ah * K, K * 4);
                         ls_prefetch_row(M.nbr + (size_t)ah * K, K * 4);
                     }
-                    const int f = ls_first_may_move(I, M, n, K, clear, al, pp);
+                    const int f = ls_first_may_move(M, n, K, clear, al, pp);
                     if (clear && lane < f) M.dlb[al] = 1;   // examined, no move
                     __syncwarp();
                     if (f == 32) { p += 32; continue; }
@@ -753,29 +752,13 @@ __device__ __forceinline__ LsMem ls_shared_full(const DevInst &I, unsigned char 
     return M;
 }
 
-// arrays in `sm` (smem_bytes) where they fit, else `fallback`; one warp
-// (copy = false: the same pointers without filling the coordinates)
-__device__ __forceinline__ LsMem ls_shared(const DevInst &I, int32_t *tour, unsigned char *sm, size_t smem_bytes,
-                                           const LsMem &fallback, bool copy = true)
+// where ls_shared_full's arrays do not all fit: all but the coordinates in `sm`
+// (smem_bytes) if they do, else `fallback`
+__device__ __forceinline__ LsMem ls_shared(const DevInst &I, unsigned char *sm, size_t smem_bytes, const LsMem &fallback)
 {
-    const int n = I.n;
-    if (ls_smem_core(n) > smem_bytes) return fallback;
-    LsMem M;
-    M.tour = reinterpret_cast<int32_t *>(sm);
-    M.pos = reinterpret_cast<int32_t *>(sm + (size_t)n * 4);
-    M.el = reinterpret_cast<float *>(sm + (size_t)n * 8);
-    M.dlb = sm + (size_t)n * 12;
+    if (ls_smem_core(I.n) > smem_bytes) return fallback;
+    LsMem M = ls_shared_full(I, sm);
     M.xy = reinterpret_cast<const float2 *>(I.xy);
-    M.nbr = I.nbr;
-    M.nbrd32 = I.nbrd32;
-    if (I.kind == 0 && ls_smem_full(n) <= smem_bytes) {
-        float2 *sxy = reinterpret_cast<float2 *>(sm + ls_xy_offset(n));
-        if (copy) {
-            for (int p = threadIdx.x & 31; p < n; p += 32) sxy[p] = reinterpret_cast<const float2 *>(I.xy)[p];
-            __syncwarp();
-        }
-        M.xy = sxy;
-    }
     return M;
 }
 
