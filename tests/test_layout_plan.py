@@ -86,6 +86,8 @@ def plan(tmp_path_factory):
     (0, 2, [(36, 1000, 64, 20, 0)], 16),
     (0, 3, [(16, 1000, 64, 20, 0)], 8),                              # 15 clusters of 8 fit
     (2, 3, [(128, 500, 32, 20, 0)], 4),
+    (0, 0, [(1000, 12, 4, 8, 0)], 2),                                # seven share an SM
+    (0, 0, [(3000, 40, 10, 8, 0)], 1),
 ])
 def test_block_width(plan, apw, clog, parts, block):
     st, groups = plan(apw, clog, parts)
