@@ -535,7 +535,8 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
     // where their shared memory does (128 x n = 1000, m = 64 per iteration: on
     // clusters of 8 2.09 ms with 8 warps a CTA and 1.13 with 4; 256 x n = 1000 on one
     // SM each, no room for two: 1.31 ms with 8, 1.22 with 16; 1000 x n = 12 37.3 us with
-    // 4, 25.5 with 2).  On a cluster no fewer than 4: its CTA 0 selects alone while
+    // 4, 25.5 with 2; 128 x n = 500, m = 32 with 32 ants per warp, one warp of them,
+    // 0.81 ms in blocks of 1, 0.56 in blocks of 16).  On a cluster no fewer than 4: its CTA 0 selects alone while
     // the others wait (128 x n = 1000 on clusters of 8: 1.32 ms with 2).
     double load = 0.0;
     for (const FusedGroup &G : groups) load += (double)G.count / dev.clusters[G.clog];
@@ -543,7 +544,7 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
         const size_t smem = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, G.apw, G.stride, G.xy_cap, G.list_rows);
         const int room = (int)(SM_SMEM / (smem + CTA_SMEM_RESERVED));
         const int share = std::max(1, std::min(std::min((int)std::ceil(load), room), G.clog ? 4 : 16));
-        G.block_warps = std::max(G.warps, G.apw > 8 ? 1 : 16 / share);
+        G.block_warps = std::max(G.warps, 16 / share);
     }
     // groups in order of their largest instance's work: the group launched
     // first gets SMs first, and the largest instances bound the batch

@@ -88,6 +88,8 @@ def plan(tmp_path_factory):
     (2, 3, [(128, 500, 32, 20, 0)], 4),
     (0, 0, [(1000, 12, 4, 8, 0)], 2),                                # seven share an SM
     (0, 0, [(3000, 40, 10, 8, 0)], 1),
+    (16, 0, [(600, 30, 8, 8, 0)], 4),
+    (32, 0, [(100, 500, 32, 20, 1)], 16),
 ])
 def test_block_width(plan, apw, clog, parts, block):
     st, groups = plan(apw, clog, parts)
