@@ -116,11 +116,10 @@ def dist_env():
 # workload under profiles/ gives the command.  Reported as roofline.traffic
 # only for the same workload and layout: the per-instance layout
 # (ants_per_warp 0) with lookup lists, smallest cluster 1.
-# NCU_TRAFFIC is the capture of the warp-segment kernel, kept for comparison;
-# FUSED_TRAFFIC is the same capture of the present one (one ant per lane quad).
-_T_PER_INSTANCE = (0.613120768e9 + 0.943468032e9) + (6.650183680e9 + 3.744521984e9)
-NCU_TRAFFIC = {("batch128", 1, 0, 32, 0, 200): _T_PER_INSTANCE}
-FUSED_TRAFFIC = {("batch128", 1, 0, 32, 0, 200): (0.068993024e9 + 0.027493888e9) + (13.042279424e9 + 6.701411328e9)}
+# FUSED_TRAFFIC holds the capture of the present kernel; NCU_TRAFFIC, which no
+# line reports, that of the kernel with 8 or 16 lanes per ant.
+NCU_TRAFFIC = {("batch128", 1, 0, 32, 0, 200): (0.613120768e9 + 0.943468032e9) + (6.650183680e9 + 3.744521984e9)}
+FUSED_TRAFFIC = {("batch128", 1, 0, 32, 0, 200): (0.068637952e9 + 0.027209472e9) + (13.056731648e9 + 6.711549952e9)}
 
 
 def load_peaks():
@@ -651,8 +650,9 @@ def run_ours(args):
                        "l2": "256 MiB buffer written between timed steps (L2 is 129 MB)",
                        "inputs": "resident in HBM before the timed region",
                        "ants_per_warp": (ex.ants_per_warp or
-                                         ("per instance: 4 on one CTA where table, masks and coordinates fit, "
-                                          "else 2 on a cluster" if args.fused else 4)), "fused": args.fused,
+                                         ("per instance: 8 on one CTA where table, masks and coordinates fit, "
+                                          "else 2, 4 or 8 on a cluster" if args.fused else
+                                          "1 to 8, as few as keep 8 warps on every SM")), "fused": args.fused,
                        "warps_per_block": args.wpb, "cluster_log2": args.clog, "parts": args.parts,
                        "uniform_n": args.uniform_n or None,
                        "fallback_list": args.fbl, "autotune": tune,

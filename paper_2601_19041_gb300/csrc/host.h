@@ -392,15 +392,15 @@ inline int upload_inputs(const DevInst &D, const hac_instance &in, const Sizes &
     return HAC_OK;
 }
 
-// Groups the given instances by layout: local search or none, ants per warp and cluster size (the
-// fewest CTAs whose shared memory holds the instance's share of the
-// candidate table and visited masks, at least 2^clog_min), each group ordered
-// by decreasing work.  apw = 0 stands for 8 ants per warp on one CTA where the
-// instance fits one with its coordinates, else for the smallest cluster that
-// holds it and as many ants per warp as its CTAs need (below).  8 ants per warp keep the fewest warps waiting for issue slots: 64
-// ants on one SM take 839 cycles per step at n = 500 on 8 warps and 1127 on 16;
-// 128 instances of n ~ U{500..2000} decode in 250 ms, in 263 ms with 4 ants per
-// warp on one SM and in 275 ms with 4 ants per warp on the clusters.
+// Groups the given instances by layout: local search or none, ants per warp and
+// cluster size (the fewest CTAs whose shared memory holds the instance's share
+// of the candidate table and visited masks, at least 2^clog_min), each group
+// ordered by decreasing work.  apw = 0 stands for 8 ants per warp on one CTA
+// where the instance fits one with its coordinates, else for the smallest
+// cluster that holds it and as many ants per warp as its CTAs need (`adapt`
+// below).  On one SM 8 ants per warp keep the fewest warps waiting for issue
+// slots: 64 ants take 839 cycles per step at n = 500 on 8 warps and 1127 on 16;
+// 128 x n = 1000, m = 64 per iteration 0.62 ms, with 4 ants per warp 0.74.
 // `order` lists instance indices group after group.
 inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &members, int apw,
                        int clog_min, int fallback_list, const DeviceShape &dev, std::vector<FusedGroup> &groups,
@@ -417,31 +417,38 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
         if (warps > 16) return false;   // k_fused is compiled for at most 512 threads
         return fused_smem_bytes(rows, z.kp, warps, a, (z.n + 32) / 32, 0, 0) <= FUSED_SMEM_LIMIT;
     };
-    for (int q = 0; q < count; ++q) {
-        if (zs[members[q]].n > 65534) return HAC_EUNSUPPORTED;
-        int rows, warps;
-        if (apw == 0) {
-            // one CTA (one SM) whenever the table, the visited masks and the
-            // coordinates of the fallback scan fit; the lookup lists then stay
-            // in global memory unless the group's CTAs have room for them.
-            // One SM per instance instead of a cluster of two frees SMs for
-            // the rest of the batch, whose makespan is otherwise bound by the
-            // SM time of the clusters rather than by its longest instance.
-            const Sizes &z = zs[members[q]];
-            qapw[q] = 8;
-            if (clog_min == 0 && fits(q, 0, 8, rows, warps) &&
-                fused_smem_bytes(rows, z.kp, warps, 8, (z.n + 32) / 32, z.n, 0) <= FUSED_SMEM_LIMIT) {
-                clog[q] = 0;
-                continue;
+    // the cluster and ants per warp of every instance on its own; false: some instance fits none
+    auto place = [&] {
+        for (int q = 0; q < count; ++q) {
+            if (zs[members[q]].n > 65534) return false;
+            clog[q] = -1;
+            qapw[q] = apw;
+            int rows, warps;
+            if (apw == 0) {
+                // one CTA (one SM) whenever the table, the visited masks and the
+                // coordinates of the fallback scan fit; the lookup lists then stay
+                // in global memory unless the group's CTAs have room for them.
+                // One SM per instance instead of a cluster of two frees SMs for
+                // the rest of the batch, whose makespan is otherwise bound by the
+                // SM time of the clusters rather than by its longest instance.
+                const Sizes &z = zs[members[q]];
+                qapw[q] = 8;
+                if (clog_min == 0 && fits(q, 0, 8, rows, warps) &&
+                    fused_smem_bytes(rows, z.kp, warps, 8, (z.n + 32) / 32, z.n, 0) <= FUSED_SMEM_LIMIT) {
+                    clog[q] = 0;
+                    continue;
+                }
             }
+            // (apw = 0: where masks for whole warps of 8 ants do not fit, 4 or 2)
+            for (int a = qapw[q]; a && clog[q] < 0; a = apw == 0 && a > 2 ? a / 2 : 0)
+                for (int cl = clog_min; cl <= 3; ++cl)
+                    if (fits(q, cl, a, rows, warps)) { clog[q] = cl; qapw[q] = a; break; }
+            if (clog[q] < 0) return false;
         }
-        // (apw = 0: where masks for whole warps of 8 ants do not fit, 4 or 2)
-        for (int a = qapw[q]; a && clog[q] < 0; a = apw == 0 && a > 2 ? a / 2 : 0)
-            for (int cl = clog_min; cl <= 3; ++cl)
-                if (fits(q, cl, a, rows, warps)) { clog[q] = cl; qapw[q] = a; break; }
-        if (clog[q] < 0) return HAC_EUNSUPPORTED;
-    }
-    if (apw == 0) {
+        return true;
+    };
+    // layouts left open, where the instances together leave SMs idle or warps short
+    auto adapt = [&] {
         // More than 64 ants on one SM are more than 8 warps, which wait for issue
         // slots, and on a cluster more than 32 per CTA leave 8 to a warp: while SMs
         // are idle, these instances go to the largest cluster of which the device
@@ -480,53 +487,61 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
                 if (share * warps <= 8) { qapw[q] = a; break; }
             }
         }
-    }
+    };
     const int apws[5] = {2, 4, 8, 16, 32};
     auto in_group = [&](int q, int cl, int a, int ls) {
         return clog[q] == cl && qapw[q] == a && (zs[members[q]].ls != 0) == (ls != 0);
     };
-    for (;;) {   // group caps may exceed the limit when members differ: move a group up
-        groups.clear();
-        bool again = false;
-        for (int cl = 0; cl <= 3 && !again; ++cl)
-            for (int ai = 0; ai < 10 && !again; ++ai) {
-                const int a = apws[ai >> 1], ls = ai & 1;
-                FusedGroup G;
-                G.clog = cl;
-                G.apw = a;
-                G.ls = ls;
-                for (int q = 0; q < count; ++q) {
-                    if (!in_group(q, cl, a, ls)) continue;
-                    int rows, warps;
-                    fits(q, cl, a, rows, warps);
-                    const Sizes &z = zs[members[q]];
-                    G.count++;
-                    G.rows_cap = std::max(G.rows_cap, rows);
-                    G.kp_cap = std::max(G.kp_cap, z.kp);
-                    G.stride = std::max(G.stride, (z.n + 32) / 32);   // bits 0..n (n: padding)
-                    G.warps = std::max(G.warps, warps);
+    // the groups, with the caps of their members; false: some group's do not fit together
+    auto group = [&] {
+        for (;;) {   // group caps may exceed the limit when members differ: move a group up
+            groups.clear();
+            bool again = false;
+            for (int cl = 0; cl <= 3 && !again; ++cl)
+                for (int ai = 0; ai < 10 && !again; ++ai) {
+                    const int a = apws[ai >> 1], ls = ai & 1;
+                    FusedGroup G;
+                    G.clog = cl;
+                    G.apw = a;
+                    G.ls = ls;
+                    for (int q = 0; q < count; ++q) {
+                        if (!in_group(q, cl, a, ls)) continue;
+                        int rows, warps;
+                        fits(q, cl, a, rows, warps);
+                        const Sizes &z = zs[members[q]];
+                        G.count++;
+                        G.rows_cap = std::max(G.rows_cap, rows);
+                        G.kp_cap = std::max(G.kp_cap, z.kp);
+                        G.stride = std::max(G.stride, (z.n + 32) / 32);   // bits 0..n (n: padding)
+                        G.warps = std::max(G.warps, warps);
+                    }
+                    if (!G.count) continue;
+                    const size_t base = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, 0, 0);
+                    if (base > FUSED_SMEM_LIMIT) {
+                        if (cl == 3) return false;
+                        for (int q = 0; q < count; ++q) if (in_group(q, cl, a, ls)) clog[q] = cl + 1;
+                        again = true;
+                        break;
+                    }
+                    // coordinates of the fallback scan in shared memory when they still fit
+                    int nmax = 0;
+                    for (int q = 0; q < count; ++q)
+                        if (in_group(q, cl, a, ls)) nmax = std::max(nmax, zs[members[q]].n);
+                    if (base + (size_t)nmax * 8 <= FUSED_SMEM_LIMIT) G.xy_cap = nmax;
+                    // and the lookup lists of this CTA's rows
+                    if (fallback_list &&
+                        fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, G.xy_cap, G.rows_cap) <=
+                            FUSED_SMEM_LIMIT)
+                        G.list_rows = G.rows_cap;
+                    groups.push_back(G);
                 }
-                if (!G.count) continue;
-                const size_t base = fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, 0, 0);
-                if (base > FUSED_SMEM_LIMIT) {
-                    if (cl == 3) return HAC_EUNSUPPORTED;
-                    for (int q = 0; q < count; ++q) if (in_group(q, cl, a, ls)) clog[q] = cl + 1;
-                    again = true;
-                    break;
-                }
-                // coordinates of the fallback scan in shared memory when they still fit
-                int nmax = 0;
-                for (int q = 0; q < count; ++q)
-                    if (in_group(q, cl, a, ls)) nmax = std::max(nmax, zs[members[q]].n);
-                if (base + (size_t)nmax * 8 <= FUSED_SMEM_LIMIT) G.xy_cap = nmax;
-                // and the lookup lists of this CTA's rows
-                if (fallback_list &&
-                    fused_smem_bytes(G.rows_cap, G.kp_cap, G.warps, a, G.stride, G.xy_cap, G.rows_cap) <=
-                        FUSED_SMEM_LIMIT)
-                    G.list_rows = G.rows_cap;
-                groups.push_back(G);
-            }
-        if (!again) break;
+            if (!again) return true;
+        }
+    };
+    if (!place()) return HAC_EUNSUPPORTED;
+    if (apw == 0) adapt();
+    if (!group()) {   // members that share a group only since adapt(): each where it fits on its own
+        if (apw != 0 || !place() || !group()) return HAC_EUNSUPPORTED;
     }
     // Block width.  The warps beyond those that build tours share the rest of an
     // iteration; 16 fill an SM's registers, so when the batch's CTAs -- all
@@ -536,8 +551,9 @@ inline int plan_groups(const std::vector<Sizes> &zs, const std::vector<int> &mem
     // clusters of 8 2.09 ms with 8 warps a CTA and 1.13 with 4; 256 x n = 1000 on one
     // SM each, no room for two: 1.31 ms with 8, 1.22 with 16; 1000 x n = 12 37.3 us with
     // 4, 25.5 with 2; 128 x n = 500, m = 32 with 32 ants per warp, one warp of them,
-    // 0.81 ms in blocks of 1, 0.56 in blocks of 16).  On a cluster no fewer than 4: its CTA 0 selects alone while
-    // the others wait (128 x n = 1000 on clusters of 8: 1.32 ms with 2).
+    // 0.81 ms in blocks of 1, 0.56 in blocks of 16).  On a cluster no fewer than 4:
+    // its CTA 0 selects alone while the others wait (128 x n = 1000 on clusters of 8:
+    // 1.32 ms with 2).
     double load = 0.0;
     for (const FusedGroup &G : groups) load += (double)G.count / dev.clusters[G.clog];
     for (FusedGroup &G : groups) {

@@ -147,3 +147,30 @@ def test_autotuner_candidates(plan, count, step_apw):
     for apw, wpb, graph, fused, fbl, prof, clog, parts in cands:
         assert apw in (0, 1, 2, 4, 16, 32) and 0 <= wpb <= 8 and graph == 1 and fbl in (0, 32) and prof == 0
         assert fused == 0 or (apw != 1 and 0 <= clog <= 3)
+
+
+def test_members_that_do_not_fit_together_are_placed_one_by_one(plan):
+    # spread over clusters of 8, the ten with many ants would share a group with
+    # the one whose table takes a CTA's shared memory: masks of both do not fit
+    st, groups = plan(0, 0, [(1, 14000, 64, 20, 0), (10, 500, 128, 20, 0)])
+    assert st == 0 and sorted((g[0], g[1], g[2]) for g in groups) == [(1, 3, 8), (10, 0, 8)], groups
+    st, groups = plan(0, 0, [(1, 14000, 64, 20, 0)])
+    assert st == 0 and [(g[0], g[1], g[2]) for g in groups] == [(1, 3, 2)], groups
+    st, groups = plan(0, 0, [(1, 60000, 64, 20, 0)])
+    assert st != 0 and not groups
+
+
+# What fits in some layout of its own is taken by the open layout, alone and in a
+# batch, and every group stays inside the limits of a block.
+@pytest.mark.parametrize("n", [3, 40, 1000, 1700, 5000, 9000, 13000])
+def test_open_layout_takes_what_fits(plan, n):
+    for m in (1, 8, 33, 64, 65, 130, 600, 1024):
+        for k in (4, 20, 32):
+            named = [plan(a, 0, [(1, n, m, k, 0)])[0] == 0 for a in (2, 4)]
+            st, groups = plan(0, 0, [(1, n, m, k, 0)])
+            assert st == 0 or not any(named), (n, m, k)
+            for count in (1, 20, 200):
+                st2, groups = plan(0, 0, [(count, n, m, k, 0), (2, 100, 10, k, 1)])
+                assert st2 == st
+                for g in groups:
+                    assert g[3] <= g[4] <= 16 and g[5] <= 226 * 1024 and g[2] in (2, 4, 8), groups
