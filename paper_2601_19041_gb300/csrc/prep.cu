@@ -744,9 +744,10 @@ __global__ void k_nbr(const DevInst *insts, const int2 *rowmap)
 
 // The fallback of Alg. 2 happens when no candidate of the current node has a
 // positive weight.  When every candidate's choice value stays positive for
-// the whole run (alpha = 1 and fl32(tau_min * W) > 0 at the smallest bound,
-// which only grows), that means all candidates are visited, so the lookup
-// list may skip them.
+// the whole run (alpha = 1 and fl32(tau * W) > 0 at the smallest tau: the lower
+// bound, or the upper one where that is smaller, as with one candidate; both
+// only grow), that means all candidates are visited, so the lookup list may
+// skip them.
 __global__ void k_fbl_check(const DevInst *insts, const int2 *slotmap)
 {
     int2 sm = slotmap[blockIdx.x];
@@ -755,7 +756,8 @@ __global__ void k_fbl_check(const DevInst *insts, const int2 *slotmap)
     size_t s = (size_t)sm.y + threadIdx.x;
     if (s >= (size_t)I.n * I.k_pad) return;
     if (I.alpha != 1.0) { if (s == 0) I.st->fbl_unsafe = 1; return; }
-    if (I.cand[s] >= 0 && !(__fmul_rn(I.st->tau_min, I.W[s]) > 0.0f)) I.st->fbl_unsafe = 1;
+    const float tau = fminf(I.st->tau_min, I.st->tau_max);
+    if (I.cand[s] >= 0 && !(__fmul_rn(tau, I.W[s]) > 0.0f)) I.st->fbl_unsafe = 1;
 }
 
 // For the fallback of Alg. 2 (instances without a second-level list, n >
